@@ -50,6 +50,31 @@ def test_ga_step_matches_the_oracle_bit_for_bit(P, n_par, rate, bad, ties, G):
     assert np.array_equal(x_out.cpu().numpy(), oga.phenotype(want, lo, hi))
 
 
+@pytest.mark.parametrize("P,G", [(2, 6), (3, 1), (31, 6), (32, 9), (33, 6), (64, 16), (65, 6), (127, 2), (129, 6),
+                                 (255, 1), (257, 6), (1025, 9), (2049, 3), (4095, 6)])
+def test_ga_step_ranks_signed_fitness_with_ties_at_the_sort_boundaries(P, G):
+    """Populations around the sort's powers of two and the 256 genes of a CTA; fitness of both signs, zeros of
+    both signs (equal), ties and non-finite values; ranks and genes equal the oracle's bit for bit."""
+    from paper_1909_11474_gb300 import binding
+    rng = np.random.default_rng(P)
+    n_par = max(1, P // 3)
+    Z = np.round(rng.normal(0.0, 2.0, P), 1)            # many ties
+    Z[rng.integers(0, P, P // 8 + 1)] = 0.0
+    Z[rng.integers(0, P, P // 8 + 1)] = -0.0
+    for k, v in enumerate([np.nan, np.inf, -np.inf, 5e-324, -5e-324]):
+        Z[(11 * k + 1) % P] = v
+    genes = rng.uniform(0.0, 1.0, (P, G))
+    u = rng.uniform(0.0, 1.0, oga.n_uniforms(P, n_par, G))
+    want, order = oga.ga_step(Z, genes, u, n_par, 0.2)
+    d = lambda a: torch.tensor(a, dtype=torch.float64, device="cuda")
+    g_out, x_out = (torch.empty((P, G), dtype=torch.float64, device="cuda") for _ in range(2))
+    o_out = torch.empty(P, dtype=torch.int32, device="cuda")
+    binding.ga_step(d(Z), d(genes), d(u), d(np.zeros(G)), d(np.ones(G)), n_par, 0.2, g_out, x_out, o_out)
+    assert np.array_equal(o_out.cpu().numpy(), order)
+    assert np.array_equal(g_out.cpu().numpy(), want)
+    assert np.array_equal(x_out.cpu().numpy(), want)
+
+
 def test_ga_step_rejects_bad_arguments():
     from paper_1909_11474_gb300 import binding
     Z, genes, u, lo, hi = _case(1, 8, 4)
