@@ -9,6 +9,19 @@
 
 namespace tsf {
 
+// the kernels are compiled in batch_fit32.cu, batch_eval32.cu, batch_64.cu, batch_gen.cu and batch_gen64.cu
+#define TSF_EXTERN_BUCKET(R, GEN, FIT) \
+  extern template cudaError_t launch_bucket<R, GEN, FIT>(const BatchParams &, const Bucket &, bool, cudaStream_t);
+TSF_EXTERN_BUCKET(float, false, true)
+TSF_EXTERN_BUCKET(float, false, false)
+TSF_EXTERN_BUCKET(float, true, true)
+TSF_EXTERN_BUCKET(float, true, false)
+TSF_EXTERN_BUCKET(double, false, true)
+TSF_EXTERN_BUCKET(double, false, false)
+TSF_EXTERN_BUCKET(double, true, true)
+TSF_EXTERN_BUCKET(double, true, false)
+#undef TSF_EXTERN_BUCKET
+
 size_t batch_smem_bytes_pt(int precision, int nb, int nq, int nat, int ncta) {
   const bool cl = ncta > 1;
   if (precision == 64)
@@ -62,10 +75,10 @@ cudaError_t launch_batch(const Ctx &ctx, const BatchPlan &plan, const double *pa
     const unsigned blocks = (unsigned)((std::max(P, ncounters) + 255) / 256);
     if (f64)
       prep_kernel<double><<<blocks, 256, 0, s>>>(P, params, reinterpret_cast<double *>(out.consts), out.form,
-                                                 ctx.Ntot, nullptr, nullptr, out.counters, ncounters);
+                                                 out.counters, ncounters);
     else
       prep_kernel<float><<<blocks, 256, 0, s>>>(P, params, reinterpret_cast<float *>(out.consts), out.form,
-                                                ctx.Ntot, nullptr, nullptr, out.counters, ncounters);
+                                                out.counters, ncounters);
     cudaError_t e = launched(1);
     if (e != cudaSuccess) return e;
   }
@@ -87,6 +100,7 @@ cudaError_t launch_batch(const Ctx &ctx, const BatchPlan &plan, const double *pa
   bp.E = out.E;
   bp.F = out.F;
   bp.f_ld = out.f_ld;
+  bp.aw = out.aw;
   bp.W = out.W;
   bp.tE = out.tE;
   bp.tW = out.tW;
@@ -99,9 +113,8 @@ cudaError_t launch_batch(const Ctx &ctx, const BatchPlan &plan, const double *pa
   const bool timed = ctx.timer.begin(s);
   // several buckets run side by side on the context's side streams (forked from and joined back into
   // `s` by events), so one bucket's last items overlap the next bucket's first ones
-  auto runs = [&](const Bucket &b) { return b.nitems > 0 && (!out.split_only || b.adj_split); };
   int nlaunch = 0;
-  for (const Bucket &b : plan.buckets) nlaunch += runs(b);
+  for (const Bucket &b : plan.buckets) nlaunch += b.nitems > 0;
   const bool fork = nlaunch > 1 && ensure_side(ctx, (int)plan.buckets.size()) == cudaSuccess;
   if (fork) {
     cudaError_t e = cudaEventRecord(ctx.side_ev[0], s);
@@ -112,30 +125,18 @@ cudaError_t launch_batch(const Ctx &ctx, const BatchPlan &plan, const double *pa
   for (const Bucket &b : plan.buckets) {
     const int k = bi;
     bp.counter = out.counters + bi++;
-    if (!runs(b)) continue;
+    if (b.nitems == 0) continue;
     bp.recs = plan.items.as<CtaRec>() + b.item_off;
     cudaError_t e = cudaSuccess;
     const cudaStream_t bs = s;
     cudaStream_t s = fork ? ctx.side[k % ctx.side.size()] : bs;
-    const bool cl = b.cluster > 1;
-    if (out.form == kFormTersoff) {
-      e = launch_bucket_tersoff_form(bp, b, f64, out.pdl, s);
-    } else if (!f64) {
-      const bool tuned = b.tune_P == P && b.tune_mode == mode;
-      if (!cl && b.mmax <= 4 && tuned && b.tune_pt == 16 && b.smem16 > 0)
-        e = launch_variant<16, 4, false, 3, float>(bp, b, out.pdl, s);
-      else if (!cl && b.mmax <= 4 && tuned && b.tune_nw == 12 && b.smem12 > 0)
-        e = launch_variant<kPT, 4, false, 2, float, 12>(bp, b, out.pdl, s);
-      else if (!cl && b.mmax <= 4) e = launch_variant<kPT, 4, false, 2, float>(bp, b, out.pdl, s);
-      else if (!cl && b.mmax <= 6) e = launch_variant<kPT, 6, false, 2, float>(bp, b, out.pdl, s);
-      else if (!cl) e = launch_variant<kPT, 8, false, 2, float>(bp, b, out.pdl, s);
-      else if (b.mmax <= 4) e = launch_variant<kPT, 4, true, 2, float>(bp, b, out.pdl, s);
-      else if (b.mmax <= 6) e = launch_variant<kPT, 6, true, 2, float>(bp, b, out.pdl, s);
-      else e = launch_variant<kPT, 8, true, 2, float>(bp, b, out.pdl, s);
-    } else {
-      if (!cl) e = launch_variant<kPT, 8, false, 1, double>(bp, b, out.pdl, s);
-      else e = launch_variant<kPT, 8, true, 1, double>(bp, b, out.pdl, s);
-    }
+    const bool gen = out.form == kFormTersoff, fit = mode == kModeFitness;
+    if (f64)
+      e = gen ? (fit ? launch_bucket<double, true, true>(bp, b, out.pdl, s) : launch_bucket<double, true, false>(bp, b, out.pdl, s))
+              : (fit ? launch_bucket<double, false, true>(bp, b, out.pdl, s) : launch_bucket<double, false, false>(bp, b, out.pdl, s));
+    else
+      e = gen ? (fit ? launch_bucket<float, true, true>(bp, b, out.pdl, s) : launch_bucket<float, true, false>(bp, b, out.pdl, s))
+              : (fit ? launch_bucket<float, false, true>(bp, b, out.pdl, s) : launch_bucket<float, false, false>(bp, b, out.pdl, s));
     if (e != cudaSuccess) return e;
   }
   if (fork) {
@@ -302,28 +303,14 @@ cudaError_t launch_fitness_finalize(int P, int C, const double *part, const doub
   return e;
 }
 
-// Force the module loading of every kernel the minimal-form fitness path launches (with lazy loading the
-// driver would otherwise load each on its first launch, allocating device memory for its code then).
-template <int PTV, int MMAX, bool CLUSTER, int MINB, typename R, int NW = kNW>
-static cudaError_t touch_variant() {
-  cudaFuncAttributes fa;
-  return cudaFuncGetAttributes(&fa, batch_kernel<PTV, MMAX, CLUSTER, MINB, R, NW, false>);
-}
+// Module loading of every kernel the minimal-form fitness path launches.
 cudaError_t preload_fitness_kernels() {
   cudaFuncAttributes fa;
   cudaError_t e = cudaFuncGetAttributes(&fa, prep_kernel<float>);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, prep_kernel<double>);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fitness_finalize_kernel);
-  if (e == cudaSuccess) e = touch_variant<16, 4, false, 3, float>();
-  if (e == cudaSuccess) e = touch_variant<kPT, 4, false, 2, float, 12>();
-  if (e == cudaSuccess) e = touch_variant<kPT, 4, false, 2, float>();
-  if (e == cudaSuccess) e = touch_variant<kPT, 6, false, 2, float>();
-  if (e == cudaSuccess) e = touch_variant<kPT, 8, false, 2, float>();
-  if (e == cudaSuccess) e = touch_variant<kPT, 4, true, 2, float>();
-  if (e == cudaSuccess) e = touch_variant<kPT, 6, true, 2, float>();
-  if (e == cudaSuccess) e = touch_variant<kPT, 8, true, 2, float>();
-  if (e == cudaSuccess) e = touch_variant<kPT, 8, false, 1, double>();
-  if (e == cudaSuccess) e = touch_variant<kPT, 8, true, 1, double>();
+  if (e == cudaSuccess) e = preload_fitness32();
+  if (e == cudaSuccess) e = preload_fitness64();
   if (e == cudaSuccess) e = preload_geometry64_kernels();
   return e;
 }
@@ -331,15 +318,19 @@ cudaError_t preload_fitness_kernels() {
 }  // namespace tsf
 
 // Debug builds (TSF_DEBUG_BOUNDS): the first out-of-range or misaligned shared-memory access of the
-// batched kernel, as {flag, site, byte offset, window size}; zeros otherwise. Clears the record.
+// batched kernels (the record of the first translation unit that has one), as {flag, site, byte offset,
+// window size}; zeros otherwise. Clears the records.
 extern "C" int tersoff_debug_bounds(unsigned *out4) {
-#ifdef TSF_DEBUG_BOUNDS
-  cudaError_t e = cudaMemcpyFromSymbol(out4, tsf::tsf_dbg, 4 * sizeof(unsigned));
-  unsigned z[4] = {0, 0, 0, 0};
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(tsf::tsf_dbg, z, sizeof(z));
-  return e == cudaSuccess ? 0 : 3;
-#else
   for (int k = 0; k < 4; ++k) out4[k] = 0;
-  return 0;
+#ifdef TSF_DEBUG_BOUNDS
+  using Take = cudaError_t (*)(unsigned *);
+  for (Take take : {tsf::debug_take_fit32, tsf::debug_take_eval32, tsf::debug_take_64, tsf::debug_take_gen,
+                    tsf::debug_take_gen64}) {
+    unsigned r[4];
+    if (take(r) != cudaSuccess) return 3;
+    if (r[0] && !out4[0])
+      for (int k = 0; k < 4; ++k) out4[k] = r[k];
+  }
 #endif
+  return 0;
 }

@@ -25,13 +25,11 @@
 
 #include "common.cuh"
 #include "ctx.hpp"
-#include "dual.cuh"
 
 namespace tsf {
 
 constexpr int kNW = 8;           // warps per CTA
 constexpr int kThreads = kNW * kWarp;
-constexpr int kNRed = 10;        // quantities of the adjoint kernel's forward reductions (adjoint.cu)
 // Quantities the batched kernel reduces per (parameter set, configuration): U, W[6] and the force sum
 // (sum |F - F*|^2, or sum |F|^2 where the configuration has no force target, to test finiteness).
 // Per-warp partials are FP32 sums over the warp's atoms; sums over warps and cluster ranks are FP64.
@@ -157,8 +155,7 @@ __device__ __forceinline__ void stage_load(const R *stage, int row, int pl, R &x
 }
 
 // The per-atom core of passes 1 and 2: from the bond geometry (unit vectors, r, 2/r, f_C, f_C', the
-// cosines of the bond pairs; R) and the parameter constants (T: R itself, or a dual number carrying
-// parameter tangents), U = sum_j f_C (f_R - b f_A), which is twice the site energy U_i of Eq. 2,
+// cosines of the bond pairs; R) and the parameter constants (T = R), U = sum_j f_C (f_R - b f_A), which is twice the site energy U_i of Eq. 2,
 // and P_ij = dU_i/dd_ij of every bond (the derivative of U_i itself, 1/2 included). INNER: every bond
 // is inside R1 (callers pass f_C = 1 and f_C' = 0 as constants, which the compiler folds away).
 //
@@ -569,8 +566,9 @@ struct BatchParams {
   unsigned wait_spins;             // polls of the staging wait before it gives up (a timeout)
   int mode;
   double *E;
-  void *F;                         // [P][Ntot][3], or [Ntot][3][f_ld] when f_ld > 0
-  int64_t f_ld;
+  void *F;                         // evaluation: F [P][Ntot][3]; gradient: v = 2 (F - F*) [Ntot][3][f_ld]
+  int64_t f_ld;                    // gradient: parameter-set stride of v and aw
+  float *aw;                       // gradient: [C][7][f_ld] weights a_e, a_k of every (p, c)
   double *W;
   const double *tE, *tW;
   const double *tF;                // [Ntot][3]: target forces (fitness)
@@ -753,13 +751,12 @@ struct TileEnv {
   double inv_nat;
   const double *tgt;               // fitness: the configuration's targets E*, W*_1..6 (shared memory)
   uint8_t mask;
-  bool fit;
   unsigned rank, ncta;
   const unsigned *peer_stage;
   const int *peer_b0;
 };
 
-template <int PTT, int PTW, int MMAX, bool CLUSTER, typename R, int NW, bool GEN = false>
+template <int PTT, int PTW, int MMAX, bool CLUSTER, typename R, int NW, bool GEN, bool FIT>
 __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R> &env, int tile) {
   using R4 = typename Vec4<R>::T;
   constexpr int APW = kWarp / PTT;
@@ -771,7 +768,6 @@ __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R>
   const int4 *satom = env.satom;
   const int ns = env.ns, s0 = env.s0, nat = env.nat, c = env.c, cb0 = env.cb0, B0 = env.B0;
   const uint8_t mask = env.mask;
-  const bool fit = env.fit;
   const unsigned rank = env.rank, ncta = env.ncta;
   const int per = (nat + (int)ncta - 1) / (int)ncta;   // atoms per cluster rank (the schedule's split)
   (void)per;
@@ -892,30 +888,34 @@ __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R>
 #pragma unroll
     for (int k = 0; k < 3; ++k) F[k] = o[k] - r[k];
   };
-  // the force of atom li: stored (evaluation) or its residual added to sf (fitness)
+  // the force of atom li: stored (evaluation) or its residual added to sf (fitness, gradient), and in
+  // gradient mode v = 2 (F - F*) stored with the parameter sets fastest (0 without a force target)
+  auto store_v = [&](int i, R x, R y, R z) {
+    R *vo = reinterpret_cast<R *>(a.F) + (size_t)i * 3 * a.f_ld + p;
+    if (active) {
+      vo[0] = x;
+      vo[a.f_ld] = y;
+      vo[2 * a.f_ld] = z;
+    }
+  };
   auto finish = [&](int li, const R (&F)[3]) {
     const int i = s0 + li;
-    if (a.mode == kModeEval) {
+    if (!FIT && a.mode == kModeEval) {
       if (active && a.F) {
         R *Fo = reinterpret_cast<R *>(a.F);
-        if (a.f_ld > 0) {
-          const size_t o = (size_t)i * 3 * a.f_ld + p;
-          Fo[o] = F[0];
-          Fo[o + a.f_ld] = F[1];
-          Fo[o + 2 * a.f_ld] = F[2];
-        } else {
-          const size_t o = ((size_t)p * a.Ntot + i) * 3;
-          Fo[o] = F[0];
-          Fo[o + 1] = F[1];
-          Fo[o + 2] = F[2];
-        }
+        const size_t o = ((size_t)p * a.Ntot + i) * 3;
+        Fo[o] = F[0];
+        Fo[o + 1] = F[1];
+        Fo[o + 2] = F[2];
       }
     } else if (mask & 4) {
       const R4 t = sld(&stF[li], 16);
       const R ex = F[0] - t.x, ey = F[1] - t.y, ez = F[2] - t.z;
       sf += ex * ex + ey * ey + ez * ez;
+      if constexpr (!FIT) store_v(i, R(2) * ex, R(2) * ey, R(2) * ez);
     } else {
       sf += F[0] * F[0] + F[1] * F[1] + F[2] * F[2];   // finiteness of F where no residual checks it
+      if constexpr (!FIT) store_v(i, R(0), R(0), R(0));
     }
   };
   if constexpr (APW == 1 && !CLUSTER) {
@@ -1008,7 +1008,7 @@ __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R>
   if (rank == 0 && red_thread) {   // whole warps: kNSum * PTT is a multiple of 32
     const int pp = tile * PTW + rl;
     const size_t pc = (size_t)pp * a.C + c;
-    if (a.mode == kModeEval) {
+    if (!FIT && a.mode == kModeEval) {
       if (pp < a.P) {
         if (rk == 0 && a.E) a.E[pc] = T;
         if (rk >= 1 && rk <= 6 && a.W) a.W[pc * 6 + (rk - 1)] = T;
@@ -1022,6 +1022,8 @@ __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R>
       if (rk <= 6) {
         const double d = T * env.inv_nat - env.tgt[rk];
         term = d * d;
+        if (!FIT && pp < a.P)   // a_e, a_k of the gradient
+          a.aw[((size_t)c * 7 + rk) * a.f_ld + pp] = (mask & bit) ? (float)(2.0 * d * env.inv_nat) : 0.f;
       }
       if (!(mask & bit)) term = isfinite(T) ? 0.0 : T - T;
       // the six virial terms of a parameter set sit in lanes 8g+1 .. 8g+6 of one warp: a fixed xor tree
@@ -1045,7 +1047,9 @@ __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R>
 // split into nchunks chunks of chunk_tiles parameter tiles; a CTA (or cluster) claims the next item
 // from an atomic counter, stages the configuration's geometry once (single-CTA launches: one TMA
 // bulk copy per array, completed on an mbarrier) and runs the chunk's tiles.
-template <int PT, int MMAX, bool CLUSTER, int MINB, typename R, int NW = kNW, bool GEN = false>
+// FIT: fitness, a kernel of its own (the tile's code is a large share of the instruction cache); otherwise
+// evaluation or gradient by a.mode.
+template <int PT, int MMAX, bool CLUSTER, int MINB, typename R, int NW, bool GEN, bool FIT>
 __global__ void __launch_bounds__(NW * kWarp, MINB) batch_kernel(const BatchParams a) {
   using R4 = typename Vec4<R>::T;
   extern __shared__ __align__(32) unsigned char smem[];
@@ -1066,7 +1070,7 @@ __global__ void __launch_bounds__(NW * kWarp, MINB) batch_kernel(const BatchPara
     rank = cluster_ctarank();
     ncta = cluster_nctarank();
   }
-  const bool fit = a.mode == kModeFitness;
+  const bool fit = FIT || a.mode != kModeEval;   // fitness and gradient: targets and residuals
   if constexpr (!CLUSTER) {
     if (tid == 0) {
       mbar_init(&mbar, 1);
@@ -1246,7 +1250,7 @@ __global__ void __launch_bounds__(NW * kWarp, MINB) batch_kernel(const BatchPara
       peer_b0[ncta] = a.recs[rec0 + ncta - 1].B0 + a.recs[rec0 + ncta - 1].nb - cb0;
     }
 
-    const TileEnv<R> env = {stage, sA, sB, sC, satom, srev, stF, ns, s0, nat, c, cb0, B0, rec.inv_nat, s_tgt, mask, fit,
+    const TileEnv<R> env = {stage, sA, sB, sC, satom, srev, stF, ns, s0, nat, c, cb0, B0, rec.inv_nat, s_tgt, mask,
                              rank, ncta, peer_stage, peer_b0};
     pdl_wait();   // per-call constants of the preparation kernel (a no-op after the first item)
     // the last tile may hold fewer parameter sets: the FP32 single-CTA variants for up to 4 neighbours
@@ -1255,21 +1259,18 @@ __global__ void __launch_bounds__(NW * kWarp, MINB) batch_kernel(const BatchPara
     constexpr bool kNarrow = !CLUSTER && MMAX <= 4 && sizeof(R) == 4 && PT >= 16;
     for (int tile = tile0; tile < tile1; ++tile) {
       const int width = min(PT, a.P - tile * PT);
-      if (kNarrow && a.narrow && width <= 8) tile_pass<(kNarrow ? 8 : PT), PT, MMAX, CLUSTER, R, NW, GEN>(a, env, tile);
+      if (kNarrow && a.narrow && width <= 8) tile_pass<(kNarrow ? 8 : PT), PT, MMAX, CLUSTER, R, NW, GEN, FIT>(a, env, tile);
       else if (kNarrow && PT > 16 && a.narrow && width <= 16)
-        tile_pass<(kNarrow ? 16 : PT), PT, MMAX, CLUSTER, R, NW, GEN>(a, env, tile);
-      else tile_pass<PT, PT, MMAX, CLUSTER, R, NW, GEN>(a, env, tile);
+        tile_pass<(kNarrow ? 16 : PT), PT, MMAX, CLUSTER, R, NW, GEN, FIT>(a, env, tile);
+      else tile_pass<PT, PT, MMAX, CLUSTER, R, NW, GEN, FIT>(a, env, tile);
     }
   }
 }
 
 // Per call, one thread per parameter set: the FP32/FP64 constants of every parameter set (PConsts).
-// When tF4 is given (the adjoint kernel), also one thread per atom: the target forces in the working
-// precision as R4 (x, y, z, |F|^2).
 template <typename R>
 __global__ void prep_kernel(int P, const double *__restrict__ params, R *__restrict__ consts, int form,
-                            int64_t Ntot, const double *__restrict__ tF, typename Vec4<R>::T *__restrict__ tF4,
-                            int *__restrict__ counters = nullptr, int ncounters = 0) {
+                            int *__restrict__ counters, int ncounters) {
   pdl_trigger();   // the batched kernel may start staging geometry; it waits before reading our output
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < ncounters) counters[t] = 0;   // the work counters of the batched launches that follow
@@ -1308,15 +1309,6 @@ __global__ void prep_kernel(int P, const double *__restrict__ params, R *__restr
     o[13] = (R)(ga * c * c);
     o[14] = (R)(d * d);
     o[15] = (R)(ga * c * c / (d * d));
-  }
-  if (tF4 && t < Ntot) {
-    const double fx = tF[3 * t], fy = tF[3 * t + 1], fz = tF[3 * t + 2];
-    typename Vec4<R>::T v;
-    v.x = (R)fx;
-    v.y = (R)fy;
-    v.z = (R)fz;
-    v.w = (R)(fx * fx + fy * fy + fz * fz);
-    tF4[t] = v;
   }
 }
 

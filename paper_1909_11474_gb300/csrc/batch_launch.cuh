@@ -9,12 +9,11 @@ namespace tsf {
 
 constexpr int kPT = 32;   // parameter sets per warp: one atom per warp
 
-template <int PTV, int MMAX, bool CLUSTER, int MINB, typename R, int NW = kNW, bool GEN = false>
+template <int PTV, int MMAX, bool CLUSTER, int MINB, typename R, int NW, bool GEN, bool FIT>
 inline cudaError_t launch_variant(BatchParams bp, const Bucket &b, bool pdl, cudaStream_t s) {
-  auto kern = batch_kernel<PTV, MMAX, CLUSTER, MINB, R, NW, GEN>;
+  auto kern = batch_kernel<PTV, MMAX, CLUSTER, MINB, R, NW, GEN, FIT>;
   const size_t smem = PTV != kPT ? b.smem16 : NW != kNW ? b.smem12 : b.smem;
-  int gen_per_sm = 0;                              // Tersoff-form variants: occupancy queried per launch
-  int &per_sm = GEN ? gen_per_sm : PTV != kPT ? b.per_sm16 : NW != kNW ? b.per_sm12 : b.per_sm;
+  int &per_sm = b.per_sm[PTV != kPT ? 4 : NW != kNW ? 5 : 2 * (GEN ? 1 : 0) + (FIT ? 1 : 0)];
   constexpr int kThr = NW * kWarp;
   bp.ntiles = (bp.P + PTV - 1) / PTV;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -75,8 +74,57 @@ inline cudaError_t launch_variant(BatchParams bp, const Bucket &b, bool pdl, cud
 }
 
 
-// One bucket in the Tersoff form (batch_gen.cu): the default schedule of the minimal form's kernels,
-// instantiated with the Tersoff-form per-atom core.
-cudaError_t launch_bucket_tersoff_form(BatchParams bp, const Bucket &b, bool f64, bool pdl, cudaStream_t s);
+// One bucket of the plan in one precision and form (R, GEN), for the fitness (FIT) or for evaluation and
+// gradient. Instantiated in translation units of their own (batch_*.cu), which compile side by side.
+template <typename R, bool GEN, bool FIT>
+cudaError_t launch_bucket(const BatchParams &bp, const Bucket &b, bool pdl, cudaStream_t s) {
+  const bool cl = b.cluster > 1;
+  if constexpr (sizeof(R) == 8) {
+    if (!cl) return launch_variant<kPT, 8, false, 1, R, kNW, GEN, FIT>(bp, b, pdl, s);
+    return launch_variant<kPT, 8, true, 1, R, kNW, GEN, FIT>(bp, b, pdl, s);
+  } else if constexpr (GEN) {
+    if (!cl && b.mmax <= 4) return launch_variant<kPT, 4, false, 2, R, kNW, GEN, FIT>(bp, b, pdl, s);
+    if (!cl) return launch_variant<kPT, 8, false, 2, R, kNW, GEN, FIT>(bp, b, pdl, s);
+    return launch_variant<kPT, 8, true, 2, R, kNW, GEN, FIT>(bp, b, pdl, s);
+  } else {
+    if constexpr (FIT) {   // schedules that only the tuner and tersoff_set_schedule choose
+      const bool tuned = b.tune_P == bp.P && b.tune_mode == bp.mode && !cl && b.mmax <= 4;
+      if (tuned && b.tune_pt == 16 && b.smem16 > 0)
+        return launch_variant<16, 4, false, 3, R, kNW, GEN, FIT>(bp, b, pdl, s);
+      if (tuned && b.tune_nw == 12 && b.smem12 > 0)
+        return launch_variant<kPT, 4, false, 2, R, 12, GEN, FIT>(bp, b, pdl, s);
+    }
+    if (!cl && b.mmax <= 4) return launch_variant<kPT, 4, false, 2, R, kNW, GEN, FIT>(bp, b, pdl, s);
+    if (!cl && b.mmax <= 6) return launch_variant<kPT, 6, false, 2, R, kNW, GEN, FIT>(bp, b, pdl, s);
+    if (!cl) return launch_variant<kPT, 8, false, 2, R, kNW, GEN, FIT>(bp, b, pdl, s);
+    if (b.mmax <= 4) return launch_variant<kPT, 4, true, 2, R, kNW, GEN, FIT>(bp, b, pdl, s);
+    if (b.mmax <= 6) return launch_variant<kPT, 6, true, 2, R, kNW, GEN, FIT>(bp, b, pdl, s);
+    return launch_variant<kPT, 8, true, 2, R, kNW, GEN, FIT>(bp, b, pdl, s);
+  }
+}
+
+// Force the module loading of every fitness kernel of one precision in the minimal form (with lazy loading
+// the driver would load each on its first launch, allocating device memory for its code then).
+template <int PTV, int MMAX, bool CLUSTER, int MINB, typename R, int NW>
+inline cudaError_t touch_variant() {
+  cudaFuncAttributes fa;
+  return cudaFuncGetAttributes(&fa, batch_kernel<PTV, MMAX, CLUSTER, MINB, R, NW, false, true>);
+}
+#ifdef TSF_DEBUG_BOUNDS
+// Reads and clears a translation unit's bounds record (tersoff_debug_bounds).
+#define TSF_DEBUG_TAKE(name)                                                          \
+  cudaError_t name(unsigned *out4) {                                                  \
+    const unsigned z[4] = {0, 0, 0, 0};                                               \
+    cudaError_t e = cudaMemcpyFromSymbol(out4, tsf_dbg, 4 * sizeof(unsigned));        \
+    if (e == cudaSuccess) e = cudaMemcpyToSymbol(tsf_dbg, z, sizeof(z));              \
+    return e;                                                                         \
+  }
+cudaError_t debug_take_fit32(unsigned *), debug_take_eval32(unsigned *), debug_take_64(unsigned *),
+    debug_take_gen(unsigned *), debug_take_gen64(unsigned *);
+#else
+#define TSF_DEBUG_TAKE(name)
+#endif
+cudaError_t preload_fitness32();   // batch_fit32.cu
+cudaError_t preload_fitness64();   // batch_64.cu
 
 }  // namespace tsf

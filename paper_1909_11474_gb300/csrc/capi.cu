@@ -59,7 +59,7 @@ int build_plan(tersoff_ctx *ctx, int precision) {
     bool operator<(const Key &o) const { return mmax != o.mmax ? mmax < o.mmax : cl < o.cl; }
   };
   std::map<Key, std::vector<int>> groups;
-  std::map<Key, size_t> smem, adj_smem, smem16, smem12;
+  std::map<Key, size_t> smem, smem16, smem12;
   // bonds and pair slots of the atoms s0 .. s1-1 of one configuration (a0 <= s0 <= s1 <= a1), and where
   // they start (for an empty slice at the end: where the configuration's bonds end)
   auto bstart = [&](int s, int a1) { return s < a1 ? c.h_boff[s] : c.h_boff[a1 - 1] + c.h_m[a1 - 1]; };
@@ -96,7 +96,6 @@ int build_plan(tersoff_ctx *ctx, int precision) {
     smem[k] = std::max(smem[k], need);
     if (chosen == 1) {
       const int nb = bstart(a1, a1) - bstart(a0, a1), nq = qstart(a1, a1) - qstart(a0, a1);
-      adj_smem[k] = std::max(adj_smem[k], tsf::adjoint_smem_bytes(nb, nq, nat));
       if (precision == 32 && mmax == 4) {
         smem16[k] = std::max(smem16[k], tsf::batch_smem_bytes_pt16(nb, nq, nat));
         smem12[k] = std::max(smem12[k], tsf::batch_smem_bytes_nw12(nb, nq, nat));
@@ -123,10 +122,6 @@ int build_plan(tersoff_ctx *ctx, int precision) {
     b.cluster = k.cl;
     b.precision = precision;
     b.smem = smem[k];
-    b.adj_smem = adj_smem[k];
-    // the gradient of configurations spread over a cluster, or beyond the adjoint kernel's shared
-    // memory, takes the split path (evaluation, weights, tangent passes per atom slice)
-    b.adj_split = k.cl > 1 || adj_smem[k] > (size_t)optin;
     b.smem16 = (k.cl == 1 && k.mmax == 4 && precision == 32) ? smem16[k] : 0;
     b.smem12 = (k.cl == 1 && k.mmax == 4 && precision == 32) ? smem12[k] : 0;
     b.item_off = (int)recs.size();
@@ -155,8 +150,6 @@ int build_plan(tersoff_ctx *ctx, int precision) {
         q.pad = 0;
         q.inv_nat = 1.0 / (double)nat;
         recs.push_back(q);
-        if (b.adj_split)
-          b.adj_split_smem = std::max(b.adj_split_smem, tsf::adjoint_split_smem_bytes(q.nb, q.nq, q.ns));
       }
     }
     b.nitems = ((int)recs.size() - b.item_off) / k.cl;   // configurations in the bucket
@@ -356,6 +349,7 @@ int tersoff_create(tersoff_ctx **out, int device) {
   if (cudaSetDevice(device) != cudaSuccess) return TERSOFF_E_CUDA;
   tersoff_ctx *ctx = new tersoff_ctx();
   ctx->c.device = device;
+  cudaDeviceGetAttribute(&ctx->c.nsm, cudaDevAttrMultiProcessorCount, device);
   // two words: the context's status, then the last neighbour build's own
   if (ctx->c.status.ensure(2 * sizeof(unsigned)) != cudaSuccess ||
       cudaMemset(ctx->c.status.p, 0, 2 * sizeof(unsigned)) != cudaSuccess) {
@@ -378,7 +372,7 @@ void tersoff_destroy(tersoff_ctx *ctx) {
   tsf::DevBuf *bufs[] = {&c.status, &c.atom_off, &c.atom_cfg, &c.pos, &c.box, &c.counters,
                          &c.cnt, &c.nbr, &c.shift, &c.boff, &c.poff, &c.brev, &c.gA32, &c.gB32,
                          &c.gcos32, &c.gA64, &c.gB64, &c.gcos64, &c.ameta, &c.arev, &c.part, &c.dpart, &c.work,
-                         &c.tf4, &c.gpart, &c.adj_v, &c.adj_ew, &c.adj_aw, &c.adj_gsplit,
+                         &c.grad_v, &c.grad_aw, &c.grad_sum,
                          &c.plan32.items, &c.plan64.items, &c.md_pos, &c.md_cnt, &c.md_nbr,
                          &c.md_shift, &c.md_cells, &c.md_cellcnt, &c.md_Pij, &c.md_red,
                          &c.md_keys, &c.md_ke, &c.md_boxd};
@@ -782,29 +776,32 @@ int tersoff_param_grad(tersoff_ctx *ctx, const double *params, int32_t P, const 
   if (c.max_m > 8) return fail(ctx, TERSOFF_E_UNSUPPORTED, "an atom has more than 8 neighbours%s");
   if (int rc = build_plan(ctx, 32)) return rc;
   cudaSetDevice(c.device);
-  const int NG = c.form ? 27 : 18;
-  TSF_CUDA(c.part.ensure((size_t)P * c.C * 3 * sizeof(double)));
+  const int nx = c.form ? 9 : 6;
+  const tsf::GradPlan gp = tsf::grad_plan(c, P);
+  TSF_CUDA(c.part.ensure((size_t)gp.block * c.C * tsf::kResidualTerms * sizeof(double)));
   TSF_CUDA(c.dpart.ensure((size_t)c.C * 3 * sizeof(double)));
-  TSF_CUDA(c.gpart.ensure((size_t)P * c.C * NG * sizeof(double)));
-  TSF_CUDA(c.work.ensure((size_t)P * 16 * sizeof(double)));
-  TSF_CUDA(c.tf4.ensure((size_t)c.Ntot * sizeof(tsf::dvec4)));
+  TSF_CUDA(c.work.ensure((size_t)gp.block * 16 * sizeof(double)));
   TSF_CUDA(c.counters.ensure(64 * sizeof(int)));
-  {
-    // split-path workspaces: v = 2 (F - F*) [Ntot][3][ldP], E and W [P][C](1 + 6), the weights
-    // [C][7][ldP], the tangent sums of every atom slice [P][slices][NG]
-    const int64_t ldP = ((int64_t)P + 31) / 32 * 32;
-    int64_t slices = 0;
-    for (const tsf::Bucket &b : c.plan32.buckets)
-      if (b.adj_split) slices += (int64_t)b.nitems * b.cluster;
-    if (slices > 0) {
-      TSF_CUDA(c.adj_v.ensure((size_t)c.Ntot * 3 * ldP * sizeof(float)));
-      TSF_CUDA(c.adj_ew.ensure((size_t)P * c.C * 7 * sizeof(double)));
-      TSF_CUDA(c.adj_aw.ensure((size_t)c.C * 7 * ldP * sizeof(float)));
-      TSF_CUDA(c.adj_gsplit.ensure((size_t)P * slices * NG * sizeof(double)));
-    }
-  }
-  TSF_CUDA(tsf::launch_param_grad(c, params, P, tg->E, tg->W, tg->F, tg->mask, w, loss, L, dL, c.work.p, c.tf4.p,
-                                  c.part.as<double>(), c.dpart.as<double>(), c.gpart.as<double>(), S(stream)));
+  TSF_CUDA(c.grad_v.ensure((size_t)c.Ntot * 3 * gp.ldP * sizeof(float)));
+  TSF_CUDA(c.grad_aw.ensure((size_t)c.C * 7 * gp.ldP * sizeof(float)));
+  TSF_CUDA(c.grad_sum.ensure((size_t)gp.block * gp.nchunks * 3 * nx * sizeof(double)));
+  tsf::BatchOut o = {};
+  o.form = c.form;
+  o.counters = c.counters.as<int>();
+  o.consts = c.work.p;
+  o.tE = tg->E;
+  o.tW = tg->W;
+  o.tF = tg->F;
+  o.tmask = tg->mask;
+  o.part = c.part.as<double>();
+  o.dpart = c.dpart.as<double>();
+  o.pdl = c.pdl;
+  o.F = c.grad_v.p;
+  o.f_ld = gp.ldP;
+  o.aw = c.grad_aw.as<float>();
+  for (int p0 = 0; p0 < P; p0 += gp.block)
+    TSF_CUDA(tsf::launch_param_grad(c, gp, params + (size_t)p0 * nx, std::min(gp.block, P - p0), o, w, loss,
+                                    c.grad_sum.as<double>(), L + p0, dL + (size_t)p0 * nx, S(stream)));
   return TERSOFF_OK;
 }
 

@@ -117,17 +117,14 @@ struct Bucket {
   int cluster;     // CTAs per configuration (1 = no cluster)
   int precision;   // 32 or 64
   size_t smem;     // dynamic shared memory per CTA
-  size_t adj_smem; // dynamic shared memory per CTA of the adjoint kernel (FP32, single-CTA buckets)
-  bool adj_split = false;   // gradient through the split path (clusters, or beyond the adjoint's memory)
-  size_t adj_split_smem = 0;  // dynamic shared memory per CTA of the split path's tangent kernel
   bool uniform;    // every configuration of the bucket has the same atom and bond counts
   int nitems;      // configurations in the bucket
   int item_off;    // first record of the bucket (records are per configuration and cluster rank)
   size_t smem16 = 0;        // shared memory per CTA of the 16-parameter-set tile variant (0: none)
   size_t smem12 = 0;        // shared memory per CTA of the 12-warp variant (0: none)
-  mutable int per_sm = 0;   // resident CTAs per SM of the bucket's kernel variant (0: not queried yet)
-  mutable int per_sm16 = 0; // the same for the 16-parameter-set tile variant
-  mutable int per_sm12 = 0; // the same for the 12-warp variant
+  // resident CTAs per SM of the bucket's kernel variants (0: not queried yet): 2 (Tersoff form) + (fitness) of
+  // the default schedule, then the 16-parameter-set tile and the 12-warp variant
+  mutable int per_sm[6] = {0, 0, 0, 0, 0, 0};
   // schedule chosen by the autotuner for one (P, mode): work items per configuration and whether the
   // last, partly filled parameter tile runs 2 or 4 atoms per warp; otherwise the built-in heuristic
   int tune_P = 0, tune_mode = -1, tune_per_conf = 0, tune_narrow = 1, tune_pt = 32, tune_nw = 8;
@@ -175,6 +172,7 @@ struct GraphCache {
 
 struct Ctx {
   int device = 0;
+  int nsm = 0;     // multiprocessors of the device
   std::string err;
   DevBuf status;   // unsigned [2]: the context's status bits, then those of the last neighbour build alone
 
@@ -203,8 +201,8 @@ struct Ctx {
   DevBuf ameta;   // [Ntot] int: bonds kept (min(cnt, M)) | (some bond beyond R1, f_C != 1) << 16
   DevBuf arev;    // [Ntot] int4: configuration-local reverse bonds of the first 8 bonds, 16 bits each
   BatchPlan plan32, plan64;
-  DevBuf part, dpart, work, tf4, gpart;
-  DevBuf adj_v, adj_ew, adj_aw, adj_gsplit;   // split-path gradient workspaces
+  DevBuf part, dpart, work;
+  DevBuf grad_v, grad_aw, grad_sum;   // gradient: v = 2 (F - F*), weights a_e and a_k, sums of the atom chunks
 
   // --- MD state ---
   int md_N = 0, md_M = 0;
@@ -268,10 +266,10 @@ struct BatchOut {
   bool pdl = false;   // launch the batched kernels with programmatic stream serialization
   int64_t wait_spins = -1;   // polls of the staging wait before it gives up (negative: built-in bound)
   int form = 0;       // 0: minimal (6 parameters), 1: Tersoff form (9 parameters, Eq. 8, free S)
-  int64_t f_ld = 0;   // > 0: F is [Ntot][3][f_ld] (parameter sets fastest) instead of [P][Ntot][3]
-  bool split_only = false;   // launch only the buckets whose gradient takes the split path
+  int64_t f_ld = 0;   // gradient: F receives v = 2 (F - F*) as [Ntot][3][f_ld], parameter sets fastest
+  float *aw = nullptr;   // gradient: weights a_e, a_k [C][7][f_ld]
 };
-enum BatchMode { kModeEval = 0, kModeFitness = 1 };
+enum BatchMode { kModeEval = 0, kModeFitness = 1, kModeGrad = 2 };
 cudaError_t launch_batch(const Ctx &ctx, const BatchPlan &plan, const double *params, int P,
                          int mode, const BatchOut &out, cudaStream_t s);
 cudaError_t autotune_batch(const Ctx &ctx, BatchPlan &plan, const double *params, int P, int mode,
@@ -299,12 +297,16 @@ int md_nve(Ctx &c, int N, double *pos, double *vel, const double *mass, const do
            void *F, double *W, cudaStream_t s, std::string &err);
 
 // adjoint.cu
-size_t adjoint_smem_bytes(int nb, int nq, int nat);
-size_t adjoint_split_smem_bytes(int nb, int nq, int ns);   // split-path tangent kernel
-cudaError_t launch_param_grad(const Ctx &ctx, const double *params, int P, const double *tE, const double *tW,
-                              const double *tF, const uint8_t *tmask, const double *w, int loss, double *L,
-                              double *dL, void *consts, void *tf4, double *part, double *dpart, double *gpart,
-                              cudaStream_t s);
+struct GradPlan {
+  int block;      // parameter sets per launch sequence
+  int tile;       // parameter sets per tile of the tangent kernel (32, 16 or 8)
+  int64_t ldP;    // parameter-set stride of v and of the weights
+  int iters;      // atoms per warp and atom slot of a CTA
+  int nchunks;    // CTAs along the atoms
+};
+GradPlan grad_plan(const Ctx &ctx, int P);
+cudaError_t launch_param_grad(const Ctx &ctx, const GradPlan &gp, const double *params, int P, const BatchOut &o,
+                              const double *w, int loss, double *gsum, double *L, double *dL, cudaStream_t s);
 
 // plain.cu
 cudaError_t launch_plain(const Ctx &ctx, const double *params, int P, double *E, double *F, double *W,

@@ -182,3 +182,58 @@ def test_param_grad_split_path_in_the_tersoff_form():
         Lr, gr = oracle.loss_and_grad(cs, params[p], t, w=WTS, loss="sq")
         assert abs(L[p] - Lr) <= 1e-4 * abs(Lr) + 1e-9, (L[p], Lr)
         assert (np.abs(dL[p] - gr) <= GRAD_TOL * np.abs(gr).max()).all(), (dL[p], gr)
+
+
+def _ragged(seed):
+    """Cells that exercise the tangent kernel's edges: a lone atom (no bonds), a dimer (zeta = 0), strongly
+    disordered cells of 7 to 62 atoms with lists of 1 to 8 bonds, some beyond R1; atom counts that fill no
+    block of atom slots evenly."""
+    rng = np.random.default_rng(seed)
+    parts = [(np.array([[1.0, 2.0, 3.0]]), np.eye(3) * 9.0), (np.array([[0.0, 0, 0], [2.4, 0.1, 0]]), np.eye(3) * 12.0)]
+    for reps, sigma, vac in (((1, 1, 1), 0.15, 1), ((2, 2, 2), 0.3, 2), ((1, 2, 2), 0.25, 0), ((2, 2, 1), 0.2, 3)):
+        pos, box = I.diamond_supercell(reps)
+        pos = pos[np.sort(rng.choice(len(pos), len(pos) - vac, replace=False))]
+        parts.append((pos + rng.normal(0, sigma, pos.shape), box))
+    return I.pack_configs(*zip(*parts))
+
+
+@pytest.mark.parametrize("form", [0, 1])
+@pytest.mark.parametrize("P", [1, 7, 8, 13, 16, 17, 24, 33])
+def test_param_grad_tiles_and_list_lengths(P, form):
+    """Every tile width of the tangent kernel (32, 16 and 8 parameter sets), full and partly filled, in both forms."""
+    from paper_1909_11474_gb300 import binding
+    cs = _ragged(3)
+    rng = np.random.default_rng(P)
+    x0 = I.TABLE2_PARAMS if form == 0 else np.array([3.2, 1.45, 2.25, 1.9, 0.65, -0.6, 0.06, 20.0, 3.0])
+    params = x0[None, :] * (1 + 0.03 * rng.normal(size=(P, len(x0))))
+    Eh, Wh, Fh = oracle.evaluate_batch(cs, x0[None, :])
+    wd = {"configs": cs, "noise": I.target_noise(rng, cs.C, cs.natoms)}
+    t = I.with_targets(wd, Eh[0] / cs.natoms, Wh[0] / cs.natoms[:, None], Fh[0], mask=np.array([7, 7, 7, 7, 3, 5], np.uint8))
+    ctx = binding.Context(0)
+    ctx.set_form(form)
+    pos, box = to_device(cs)
+    ctx.build_neighbors(cs.atom_off, pos, box, 2.8, 3.2, 16)
+    assert 5 <= ctx.build_info()[2] <= 8
+    L, dL = ctx.param_grad(torch.tensor(params, device="cuda"), targets_to_device(t), w=WTS, loss=0)
+    torch.cuda.synchronize()
+    assert ctx.get_status() == 0
+    L, dL = L.cpu().numpy(), dL.cpu().numpy()
+    for p in sorted({0, P // 2, P - 1}):
+        Lr, gr = oracle.loss_and_grad(cs, params[p], t, w=WTS, loss="sq")
+        assert abs(L[p] - Lr) <= 1e-4 * abs(Lr) + 1e-9
+        assert (np.abs(dL[p] - gr) <= GRAD_TOL * np.abs(gr).max()).all(), (dL[p], gr)
+
+
+def test_param_grad_in_blocks_of_parameter_sets():
+    """A population whose v would exceed the 1 GiB workspace is taken in blocks: the rows of every block equal
+    those of a call on them alone (same tile width, so the same arithmetic but for the sums' chunks)."""
+    ctx, cs, t, params = _setup(P=9, C=100, masks=[7] * 100, near=0.02)
+    P = 14100
+    rng = np.random.default_rng(5)
+    x = torch.tensor(params[rng.integers(0, 9, P)] * (1 + 0.01 * rng.normal(size=(P, 6))), device="cuda")
+    tg = targets_to_device(t)
+    L, dL = ctx.param_grad(x, tg, w=WTS, loss=0)
+    for a, b in ((0, 32), (13952, 14048), (P - 64, P)):
+        L1, dL1 = ctx.param_grad(x[a:b].contiguous(), tg, w=WTS, loss=0)
+        assert torch.allclose(L[a:b], L1, rtol=1e-6, atol=0)
+        assert ((dL[a:b] - dL1).abs() <= GRAD_TOL * dL1.abs().amax(1, keepdim=True)).all()
