@@ -598,7 +598,7 @@ __host__ __device__ inline size_t batch_smem(int nb, int nq, int nat, int ncta) 
   b += ((size_t)nq * sizeof(R) + 31) / 32 * 32;
   b += (size_t)nat * sizeof(int4);
   b += (size_t)nat * sizeof(R4);
-  b += (size_t)nat * sizeof(int4);
+  b += (size_t)nat * sizeof(int4) * (CLUSTER ? 2 : 1);   // reverse rows (rev_words, at most 2)
   return b;
 }
 
@@ -628,33 +628,59 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned by
 }
 constexpr unsigned kMbarSpins = 1u << 22;   // bound of a wait for one configuration's copies
 
-// Single-CTA kernels of up to four neighbours with one atom per warp keep each atom's reverse rows as
-// byte offsets in the stage (set when the item is staged), so the gather adds them to its base.
-template <int PTT, int MMAX, bool CLUSTER, typename R>
-__host__ __device__ constexpr bool kRevBytes() {
-  return PTT == 32 && MMAX <= 4 && !CLUSTER;
+// How an atom's reverse rows are kept in shared memory (srev): configuration-local bond indices, 16 bits each,
+// for up to eight bonds; byte offsets in the stage of the first four (single-CTA kernels of up to four
+// neighbours with one atom per warp: the gather adds them to its base); or, in a cluster, the shared::cluster
+// addresses of the rows in the CTAs that hold them, one int4 per four bonds.
+enum RevKind { kRevIndex = 0, kRevBytes = 1, kRevCluster = 2 };
+template <int PTT, int MMAX, bool CLUSTER>
+__host__ __device__ constexpr RevKind rev_kind() {
+  return CLUSTER ? kRevCluster : (PTT == 32 && MMAX <= 4 ? kRevBytes : kRevIndex);
+}
+// int4 of srev per atom
+template <int MMAX, bool CLUSTER>
+__host__ __device__ constexpr int rev_words() {
+  return CLUSTER && MMAX > 4 ? 2 : 1;
 }
 
-// Pass 3 of one atom with a compile-time neighbour count M from a single-CTA stage: F_i = sum_j P_ij
-// over the atom's own rows minus sum_j P_ji over the rows of the reverse bonds. rv: the reverse bonds'
-// configuration-local indices, 16 bits each (roff maps them to stage rows). Every gather forms the two
+// Pass 3 of one atom with a compile-time neighbour count M: F_i = sum_j P_ij over the atom's own rows minus
+// sum_j P_ji over the rows of the reverse bonds (in a cluster, rows of the peers' stages). Every gather forms the two
 // sums separately, each over its rows in order, and subtracts them once (F = Fo - Fr), so that an
 // atom's force has the same rounding on every path; the rows are loaded before any is summed.
 template <int M, int PTT, typename R>
 struct GatherRows {
   R o[M][3], r[M][3];
 };
-// REVB: rv holds the reverse rows' byte offsets in the stage (first four bonds; kernels of up to four
-// neighbours), otherwise their configuration-local indices, 16 bits each (roff maps them to stage rows).
-template <int M, int PTT, typename R, bool REVB>
-__device__ __forceinline__ void gather_load(const R *__restrict__ stage, int4 rv, int lb, int roff, int pl,
+// rw: the atom's srev words (RevKind KIND; roff maps bond indices to stage rows).
+template <int MMAX, bool CLUSTER>
+__device__ __forceinline__ void rev_load(const int4 *srev, int li, int (&rw)[4 * rev_words<MMAX, CLUSTER>()]) {
+  constexpr int W = rev_words<MMAX, CLUSTER>();
+#pragma unroll
+  for (int k = 0; k < W; ++k) {
+    const int4 v = sld(&srev[li * W + k], 12);
+    rw[4 * k] = v.x; rw[4 * k + 1] = v.y; rw[4 * k + 2] = v.z; rw[4 * k + 3] = v.w;
+  }
+}
+template <int M, int PTT, typename R, RevKind KIND, int NREV>
+__device__ __forceinline__ void gather_load(const R *__restrict__ stage, const int (&rw)[NREV], int lb, int roff, int pl,
                                             GatherRows<M, PTT, R> &g) {
-  const int rw[4] = {rv.x, rv.y, rv.z, rv.w};
 #pragma unroll
   for (int e = 0; e < M; ++e) stage_load<PTT, R>(stage, lb + e, pl, g.o[e][0], g.o[e][1], g.o[e][2], 13);
 #pragma unroll
   for (int e = 0; e < M; ++e) {
-    if constexpr (REVB) {
+    if constexpr (KIND == kRevCluster) {
+      static_assert(M <= NREV, "one address per bond");
+      const unsigned row = (unsigned)rw[e];
+      if constexpr (stage_packed<PTT, R>()) {
+        const float2 xy = ld_cluster2(row + pl * sizeof(float2));
+        g.r[e][0] = xy.x;
+        g.r[e][1] = xy.y;
+        g.r[e][2] = ld_cluster(row + (2 * PTT + pl) * sizeof(R), R(0));
+      } else {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) g.r[e][k] = ld_cluster(row + (k * PTT + pl) * sizeof(R), R(0));
+      }
+    } else if constexpr (KIND == kRevBytes) {
       static_assert(M <= 4, "byte offsets of the first four reverse rows");
       const R *st = reinterpret_cast<const R *>(reinterpret_cast<const unsigned char *>(stage) + rw[e]);
       stage_load_row<PTT, R>(st, pl, g.r[e][0], g.r[e][1], g.r[e][2], 15);
@@ -678,54 +704,52 @@ __device__ __forceinline__ void gather_sum(const GatherRows<M, PTT, R> &g, R &Fx
   Fy = o[1] - r[1];
   Fz = o[2] - r[2];
 }
-template <int M, int PTT, typename R, bool REVB>
-__device__ __forceinline__ void gather_atom(const R *__restrict__ stage, int4 rv, int lb, int roff, int pl,
+template <int M, int PTT, typename R, RevKind KIND, int NREV>
+__device__ __forceinline__ void gather_atom(const R *__restrict__ stage, const int (&rw)[NREV], int lb, int roff, int pl,
                                             R &Fx, R &Fy, R &Fz) {
   GatherRows<M, PTT, R> g;
-  gather_load<M, PTT, R, REVB>(stage, rv, lb, roff, pl, g);
+  gather_load<M, PTT, R, KIND, NREV>(stage, rw, lb, roff, pl, g);
   gather_sum<M, PTT, R>(g, Fx, Fy, Fz);
 }
 // Two atoms of the same neighbour count M, their loads issued together (one warp keeps both atoms'
 // rows in flight); each atom's arithmetic is that of gather_atom.
-template <int M, int PTT, typename R, bool REVB>
-__device__ __forceinline__ void gather_atom_pair(const R *__restrict__ stage, int4 rv0, int lb0, int4 rv1, int lb1,
-                                                 int roff, int pl, R (&F0)[3], R (&F1)[3]) {
+template <int M, int PTT, typename R, RevKind KIND, int NREV>
+__device__ __forceinline__ void gather_atom_pair(const R *__restrict__ stage, const int (&rw0)[NREV], int lb0,
+                                                 const int (&rw1)[NREV], int lb1, int roff, int pl, R (&F0)[3],
+                                                 R (&F1)[3]) {
   GatherRows<M, PTT, R> g0, g1;
-  gather_load<M, PTT, R, REVB>(stage, rv0, lb0, roff, pl, g0);
-  gather_load<M, PTT, R, REVB>(stage, rv1, lb1, roff, pl, g1);
+  gather_load<M, PTT, R, KIND, NREV>(stage, rw0, lb0, roff, pl, g0);
+  gather_load<M, PTT, R, KIND, NREV>(stage, rw1, lb1, roff, pl, g1);
   gather_sum<M, PTT, R>(g0, F0[0], F0[1], F0[2]);
   gather_sum<M, PTT, R>(g1, F1[0], F1[1], F1[2]);
 }
-// Dispatch on the atom's neighbour count; false when it exceeds MMAX (the caller's loop handles it).
-template <int PTT, int MMAX, typename R, bool REVB>
-__device__ __forceinline__ bool gather_dispatch(int m, const R *stage, int4 rv, int lb, int roff, int pl, R &Fx,
-                                                R &Fy, R &Fz) {
-#define TSF_GCASE(MM)                                                              \
-  case MM:                                                                         \
-    if constexpr (MMAX >= MM) {                                                    \
-      gather_atom<MM, PTT, R, REVB>(stage, rv, lb, roff, pl, Fx, Fy, Fz);          \
-      return true;                                                                 \
-    }                                                                              \
-    return false;
+// Dispatch on the atom's neighbour count; nothing for an atom without bonds (or with more than MMAX, which
+// pass 1 flagged).
+template <int PTT, int MMAX, typename R, RevKind KIND, int NREV>
+__device__ __forceinline__ void gather_dispatch(int m, const R *stage, const int (&rw)[NREV], int lb, int roff, int pl,
+                                                R (&F)[3]) {
+#define TSF_GCASE(MM)                                                                                       \
+  case MM:                                                                                                  \
+    if constexpr (MMAX >= MM) gather_atom<MM, PTT, R, KIND, NREV>(stage, rw, lb, roff, pl, F[0], F[1], F[2]); \
+    break;
   switch (m) {
-    case 0:
-      return true;
     TSF_GCASE(1) TSF_GCASE(2) TSF_GCASE(3) TSF_GCASE(4) TSF_GCASE(5) TSF_GCASE(6) TSF_GCASE(7) TSF_GCASE(8)
     default:
-      return false;
+      break;
   }
 #undef TSF_GCASE
 }
 // Both atoms with neighbour count m; false when m is not a count with a pair variant.
-template <int PTT, int MMAX, typename R, bool REVB>
-__device__ __forceinline__ bool gather_pair_dispatch(int m, const R *stage, int4 rv0, int lb0, int4 rv1, int lb1,
-                                                     int roff, int pl, R (&F0)[3], R (&F1)[3]) {
-#define TSF_PCASE(MM)                                                                    \
-  case MM:                                                                               \
-    if constexpr (MMAX >= MM) {                                                          \
-      gather_atom_pair<MM, PTT, R, REVB>(stage, rv0, lb0, rv1, lb1, roff, pl, F0, F1);   \
-      return true;                                                                       \
-    }                                                                                    \
+template <int PTT, int MMAX, typename R, RevKind KIND, int NREV>
+__device__ __forceinline__ bool gather_pair_dispatch(int m, const R *stage, const int (&rw0)[NREV], int lb0,
+                                                     const int (&rw1)[NREV], int lb1, int roff, int pl, R (&F0)[3],
+                                                     R (&F1)[3]) {
+#define TSF_PCASE(MM)                                                                                    \
+  case MM:                                                                                               \
+    if constexpr (MMAX >= MM) {                                                                          \
+      gather_atom_pair<MM, PTT, R, KIND, NREV>(stage, rw0, lb0, rw1, lb1, roff, pl, F0, F1);             \
+      return true;                                                                                       \
+    }                                                                                                    \
     return false;
   switch (m) {
     TSF_PCASE(3) TSF_PCASE(4)
@@ -745,15 +769,13 @@ struct TileEnv {
   const typename Vec4<R>::T *sA, *sB;
   const R *sC;
   const int4 *satom;
-  const int4 *srev;                // per atom: the reverse bonds' configuration-local indices, 16 bits each
+  const int4 *srev;                // per atom: the reverse rows (RevKind)
   const typename Vec4<R>::T *stF;
   int ns, s0, nat, c, cb0, B0;
   double inv_nat;
   const double *tgt;               // fitness: the configuration's targets E*, W*_1..6 (shared memory)
   uint8_t mask;
   unsigned rank, ncta;
-  const unsigned *peer_stage;
-  const int *peer_b0;
 };
 
 template <int PTT, int PTW, int MMAX, bool CLUSTER, typename R, int NW, bool GEN, bool FIT>
@@ -766,16 +788,9 @@ __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R>
   const R4 *sA = env.sA, *sB = env.sB, *stF = env.stF;
   const R *sC = env.sC;
   const int4 *satom = env.satom;
-  const int ns = env.ns, s0 = env.s0, nat = env.nat, c = env.c, cb0 = env.cb0, B0 = env.B0;
+  const int ns = env.ns, s0 = env.s0, c = env.c, cb0 = env.cb0, B0 = env.B0;
   const uint8_t mask = env.mask;
   const unsigned rank = env.rank, ncta = env.ncta;
-  const int per = (nat + (int)ncta - 1) / (int)ncta;   // atoms per cluster rank (the schedule's split)
-  (void)per;
-  const unsigned *peer_stage = env.peer_stage;
-  const int *peer_b0 = env.peer_b0;
-  (void)B0;
-  (void)peer_stage;
-  (void)peer_b0;
   (void)rank;
   (void)ncta;
   const int p = tile * PTW + pl;
@@ -833,57 +848,24 @@ __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R>
 
   // ---- pass 3: F_i = sum_j (P_ij - P_ji)
   R sf = R(0);   // sum |F - F*|^2 over the warp's atoms, or sum |F|^2 without a force target
-  // F of atom li with a neighbour count beyond the compile-time gathers (and in the cluster and
-  // several-atoms-per-warp variants): the own and the reverse rows summed in order, as in gather_sum
+  // F of atom li in the variants with several atoms in a warp: the own and the reverse rows summed in order,
+  // as in gather_sum
   auto gather_loop = [&](int li, const int4 &at, R (&F)[3]) {
     const int m = at.z, lb = at.x;
     R o[3] = {R(0), R(0), R(0)}, r[3] = {R(0), R(0), R(0)};
     for (int e = 0; e < m; ++e) {
-      {
-        R x, y, z;
-        stage_load<PTT, R>(stage, lb + e, pl, x, y, z, 13);
-        o[0] += x;
-        o[1] += y;
-        o[2] += z;
-      }
-      int packed;  // configuration-local indices of the reverse entry (bits 0-15) and of atom j (16-31)
+      R x, y, z;
+      stage_load<PTT, R>(stage, lb + e, pl, x, y, z, 13);
+      o[0] += x;
+      o[1] += y;
+      o[2] += z;
+      int packed;  // configuration-local index of the reverse entry in bits 0-15
       if constexpr (sizeof(R) == 4) packed = __float_as_int((float)sld(&sB[lb + e].w, 14));
       else packed = (int)sld(&sB[lb + e].w, 14);
-      const int rb = packed & 0xffff;
-      if constexpr (CLUSTER) {
-        // the reverse entry belongs to atom j, whose rank is its slice of the configuration's atoms
-        const unsigned rk = min((unsigned)(packed >> 16) / (unsigned)per, ncta - 1);
-        // a reverse bond outside the configuration's bond range is an inconsistent schedule:
-        // flag it and skip the peer read rather than touch another CTA's shared memory
-        if (rb < peer_b0[rk] || rb >= peer_b0[rk + 1]) {
-          set_status(a.status, TERSOFF_STATUS_NBR_OVERFLOW);
-#ifdef TSF_DEBUG_BOUNDS
-          if (atomicCAS(&tsf_dbg[0], 0u, 1u) == 0u) {
-            tsf_dbg[1] = 21;
-            tsf_dbg[2] = (unsigned)rb;
-            tsf_dbg[3] = (unsigned)peer_b0[ncta];
-          }
-#endif
-          continue;
-        }
-        const unsigned row = peer_stage[rk] + (unsigned)((rb - peer_b0[rk]) * stage_stride<PTT>() * sizeof(R));
-        if constexpr (stage_packed<PTT, R>()) {
-          const float2 xy = ld_cluster2(row + pl * sizeof(float2));
-          r[0] += xy.x;
-          r[1] += xy.y;
-          r[2] += ld_cluster(row + (2 * PTT + pl) * sizeof(R), R(0));
-        } else {
-          r[0] += ld_cluster(row + pl * sizeof(R), R(0));
-          r[1] += ld_cluster(row + (PTT + pl) * sizeof(R), R(0));
-          r[2] += ld_cluster(row + (2 * PTT + pl) * sizeof(R), R(0));
-        }
-      } else {
-        R x, y, z;
-        stage_load<PTT, R>(stage, rb + cb0 - B0, pl, x, y, z, 15);
-        r[0] += x;
-        r[1] += y;
-        r[2] += z;
-      }
+      stage_load<PTT, R>(stage, (packed & 0xffff) + cb0 - B0, pl, x, y, z, 15);
+      r[0] += x;
+      r[1] += y;
+      r[2] += z;
     }
 #pragma unroll
     for (int k = 0; k < 3; ++k) F[k] = o[k] - r[k];
@@ -918,28 +900,30 @@ __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R>
       if constexpr (!FIT) store_v(i, R(0), R(0), R(0));
     }
   };
-  if constexpr (APW == 1 && !CLUSTER) {
+  if constexpr (APW == 1) {
     // one atom per warp: two atoms (li and li + NW) per iteration, whose row loads are issued together;
     // sf still takes the warp's atoms in ascending order
+    constexpr RevKind kKind = rev_kind<PTT, MMAX, CLUSTER>();
+    constexpr int kNRev = 4 * rev_words<MMAX, CLUSTER>();
     const int roff = cb0 - B0;
     for (int l0 = warp; l0 < ns; l0 += 2 * NW) {
       const int l1 = l0 + NW;
-      const int4 at0 = sld(&satom[l0], 12), rv0 = sld(&env.srev[l0], 12);
+      const int4 at0 = sld(&satom[l0], 12);
+      int rw0[kNRev], rw1[kNRev];
+      rev_load<MMAX, CLUSTER>(env.srev, l0, rw0);
       R F0[3] = {R(0), R(0), R(0)}, F1[3] = {R(0), R(0), R(0)};   // an atom without bonds keeps F = 0
       if (l1 < ns) {
-        const int4 at1 = sld(&satom[l1], 12), rv1 = sld(&env.srev[l1], 12);
-        if (!(at0.z == at1.z &&
-              gather_pair_dispatch<PTT, MMAX, R, kRevBytes<PTT, MMAX, CLUSTER, R>()>(at0.z, stage, rv0, at0.x, rv1, at1.x, roff, pl, F0, F1))) {
-          if (!gather_dispatch<PTT, MMAX, R, kRevBytes<PTT, MMAX, CLUSTER, R>()>(at0.z, stage, rv0, at0.x, roff, pl, F0[0], F0[1], F0[2]))
-            gather_loop(l0, at0, F0);
-          if (!gather_dispatch<PTT, MMAX, R, kRevBytes<PTT, MMAX, CLUSTER, R>()>(at1.z, stage, rv1, at1.x, roff, pl, F1[0], F1[1], F1[2]))
-            gather_loop(l1, at1, F1);
+        const int4 at1 = sld(&satom[l1], 12);
+        rev_load<MMAX, CLUSTER>(env.srev, l1, rw1);
+        if (!(at0.z == at1.z && gather_pair_dispatch<PTT, MMAX, R, kKind, kNRev>(at0.z, stage, rw0, at0.x, rw1, at1.x, roff,
+                                                                          pl, F0, F1))) {
+          gather_dispatch<PTT, MMAX, R, kKind, kNRev>(at0.z, stage, rw0, at0.x, roff, pl, F0);
+          gather_dispatch<PTT, MMAX, R, kKind, kNRev>(at1.z, stage, rw1, at1.x, roff, pl, F1);
         }
         finish(l0, F0);
         finish(l1, F1);
       } else {
-        if (!gather_dispatch<PTT, MMAX, R, kRevBytes<PTT, MMAX, CLUSTER, R>()>(at0.z, stage, rv0, at0.x, roff, pl, F0[0], F0[1], F0[2]))
-          gather_loop(l0, at0, F0);
+        gather_dispatch<PTT, MMAX, R, kKind, kNRev>(at0.z, stage, rw0, at0.x, roff, pl, F0);
         finish(l0, F0);
       }
     }
@@ -1170,8 +1154,38 @@ __global__ void __launch_bounds__(NW * kWarp, MINB) batch_kernel(const BatchPara
       for (int t = tid; t < ns; t += (NW * kWarp)) {
         const int am = a.ameta[s0 + t];
         sst(&satom[t], make_int4(a.boff[s0 + t] - B0, a.poff[s0 + t] - Q0, am & 0xffff, am >> 16), 9);
+        if constexpr (CLUSTER) {
+          // addresses of the reverse rows: the reverse entry belongs to atom j, whose rank is its slice of the
+          // configuration's atoms. One outside that rank's bonds is an inconsistent schedule: it is flagged, and
+          // the atom's own stage stands in for it rather than memory beyond a peer's
+          constexpr int W = rev_words<MMAX, true>();
+          const int m = min(am & 0xffff, 4 * W), b0 = a.boff[s0 + t];
+          const int per = (nat + (int)ncta - 1) / (int)ncta;   // atoms per rank (the schedule's split)
+          int ad[4 * W];
+#pragma unroll
+          for (int e = 0; e < 4 * W; ++e) {
+            ad[e] = (int)smem_addr(stage);
+            if (e < m) {
+              int packed;   // configuration-local indices of the reverse entry (bits 0-15) and of atom j (16-31)
+              if constexpr (sizeof(R) == 4) packed = __float_as_int((float)gB[b0 - B0 + e].w);
+              else packed = (int)gB[b0 - B0 + e].w;
+              const int rk = min((packed >> 16) / per, (int)ncta - 1);
+              const CtaRec &q = a.recs[rec0 + rk];
+              const int row = (packed & 0xffff) + cb0 - q.B0;
+              if (row >= 0 && row < q.nb) {
+                ad[e] = (int)(map_to_rank(smem_addr(stage), (unsigned)rk) + (unsigned)(row * stage_stride<PT>() * sizeof(R)));
+              } else {
+                set_status(a.status, TERSOFF_STATUS_NBR_OVERFLOW);
+                ad[e] = (int)map_to_rank(smem_addr(stage), rank);
+              }
+            }
+          }
+#pragma unroll
+          for (int k = 0; k < W; ++k)
+            sst(&srev[t * W + k], make_int4(ad[4 * k], ad[4 * k + 1], ad[4 * k + 2], ad[4 * k + 3]), 9);
+        }
         int4 rv = a.arev[s0 + t];
-        if constexpr (kRevBytes<PT, MMAX, CLUSTER, R>()) {   // rows of the full-width stage, in bytes
+        if constexpr (rev_kind<PT, MMAX, CLUSTER>() == kRevBytes) {   // rows of the full-width stage, in bytes
           const int rw[2] = {rv.x, rv.y};
           int off[4];
 #pragma unroll
@@ -1179,7 +1193,7 @@ __global__ void __launch_bounds__(NW * kWarp, MINB) batch_kernel(const BatchPara
             off[e] = (((rw[e >> 1] >> (16 * (e & 1))) & 0xffff) + cb0 - B0) * (int)(stage_stride<PT>() * sizeof(R));
           rv = make_int4(off[0], off[1], off[2], off[3]);
         }
-        sst(&srev[t], rv, 9);
+        if constexpr (!CLUSTER) sst(&srev[t], rv, 9);
         if (fit) {   // target force in the working precision
           const double *f = a.tF + 3 * (int64_t)(s0 + t);
           const double fx = f[0], fy = f[1], fz = f[2];
@@ -1239,19 +1253,8 @@ __global__ void __launch_bounds__(NW * kWarp, MINB) batch_kernel(const BatchPara
         a.dpart[3 * c + 2] = (mask & 4) ? fsum : 0.0;
       }
     }
-    unsigned peer_stage[kMaxCluster];
-    int peer_b0[kMaxCluster + 1];
-    if constexpr (CLUSTER) {
-      const unsigned own = smem_addr(stage);
-      for (unsigned r = 0; r < ncta; ++r) {
-        peer_stage[r] = map_to_rank(own, r);
-        peer_b0[r] = a.recs[rec0 + r].B0 - cb0;
-      }
-      peer_b0[ncta] = a.recs[rec0 + ncta - 1].B0 + a.recs[rec0 + ncta - 1].nb - cb0;
-    }
-
     const TileEnv<R> env = {stage, sA, sB, sC, satom, srev, stF, ns, s0, nat, c, cb0, B0, rec.inv_nat, s_tgt, mask,
-                             rank, ncta, peer_stage, peer_b0};
+                             rank, ncta};
     pdl_wait();   // per-call constants of the preparation kernel (a no-op after the first item)
     // the last tile may hold fewer parameter sets: the FP32 single-CTA variants for up to 4 neighbours
     // run it with more atoms in a warp (tiles of 16 or 8 parameter sets); other variants keep the

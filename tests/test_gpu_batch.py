@@ -364,3 +364,29 @@ def test_large_cells_in_clusters_eval(ctx, precision):
     clusters = sorted({b["cluster"] for b in ctx.schedule_info(precision)})
     print("cluster sizes", clusters)
     assert max(clusters) >= 8
+
+
+@pytest.mark.parametrize("precision", [32, 64])
+@pytest.mark.parametrize("reps,vac,sigma", [((3, 2, 2), 1, 0.30), ((4, 4, 2), 3, 0.22), ((4, 4, 4), 5, 0.27)])
+def test_cluster_gather_on_disordered_cells(precision, reps, vac, sigma):
+    """Cells spread over a cluster, whose lists of up to 8 bonds take both words of reverse-row addresses, with
+    atom counts that leave the last rank a shorter slice: E/F/W against the oracle."""
+    from paper_1909_11474_gb300 import binding
+    rng = np.random.default_rng(int(np.prod(reps)))
+    pos, box = I.diamond_supercell(reps)
+    pos = pos[np.sort(rng.choice(len(pos), len(pos) - vac, replace=False))]
+    cs = I.pack_configs([pos + rng.normal(0, sigma, pos.shape)], [box])
+    params = I.population(rng, 3)[0]
+    ctx = binding.Context(0)
+    p, b = to_device(cs)
+    ctx.build_neighbors(cs.atom_off, p, b, 2.8, 3.2, 16)
+    assert 4 < ctx.build_info()[2] <= 8
+    assert precision == 64 or ctx.schedule_info(precision)[0]["cluster"] > 1
+    E, F, W = ctx.eval(torch.tensor(params, device="cuda"), precision=precision)
+    torch.cuda.synchronize()
+    assert ctx.get_status() == 0
+    Er, Wr, Fr, ES, WS, FS = oracle.evaluate_batch(cs, params, scales=True, force_scales=True)
+    tol = TOL32 if precision == 32 else TOL64
+    assert energy_rel_err(E.cpu().numpy(), Er, ES).max() < tol["E"]
+    assert virial_rel_err(W.cpu().numpy(), Wr, WS).max() < tol["W"]
+    assert force_err(F.cpu().double().numpy(), Fr, FS) < tol["F"]
