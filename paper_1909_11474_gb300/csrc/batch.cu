@@ -25,22 +25,23 @@ TSF_EXTERN_BUCKET(double, true, false)
 size_t batch_smem_bytes_pt(int precision, int nb, int nq, int nat, int ncta) {
   const bool cl = ncta > 1;
   if (precision == 64)
-    return cl ? batch_smem<kPT, true, double>(nb, nq, nat, ncta) : batch_smem<kPT, false, double>(nb, nq, nat, 1);
+    return cl ? batch_smem<kPT64, true, double>(nb, nq, nat, ncta) : batch_smem<kPT64, false, double>(nb, nq, nat, 1);
   return cl ? batch_smem<kPT, true, float>(nb, nq, nat, ncta) : batch_smem<kPT, false, float>(nb, nq, nat, 1);
 }
-
-int batch_param_tile() { return kPT; }
 
 size_t batch_smem_bytes_pt16(int nb, int nq, int nat) { return batch_smem<16, false, float>(nb, nq, nat, 1); }
 size_t batch_smem_bytes_nw12(int nb, int nq, int nat) { return batch_smem<kPT, false, float, 12>(nb, nq, nat, 1); }
 
 static int precision_of(const BatchPlan &plan) { return plan.precision; }
 
-int batch_max_smem_optin() {
+int batch_param_tile(int precision) { return precision == 64 ? kPT64 : kPT; }
+
+// Dynamic shared memory a CTA can have beside the kernels' static part (FP64: the tables of fx64.cuh).
+int batch_max_smem_optin(int precision) {
   int dev = 0, v = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  return v;
+  return v - (precision == 64 ? (int)sizeof(FxTables) + 512 : 512);
 }
 
 // Side streams (at most kSide) and their events, created on first use.
@@ -186,7 +187,7 @@ cudaError_t autotune_batch(const Ctx &ctx, BatchPlan &plan, const double *params
     float bt = 3.4e38f;
     // variants: 32-wide tiles with 8 or 12 warps per CTA, 16-wide tiles with 8 (where they exist)
     for (int var = 0; var < 3; ++var) {
-      const int pt = var == 2 ? 16 : kPT, warps = var == 1 ? 12 : kNW;
+      const int pt = var == 2 ? 16 : batch_param_tile(precision_of(plan)), warps = var == 1 ? 12 : kNW;
       if ((var == 1 && b.smem12 == 0) || (var == 2 && b.smem16 == 0)) continue;
       const int ntiles = (P + pt - 1) / pt;
       std::vector<int> cands;

@@ -7,8 +7,8 @@ template cudaError_t launch_bucket<double, false, true>(const BatchParams &, con
 template cudaError_t launch_bucket<double, false, false>(const BatchParams &, const Bucket &, bool, cudaStream_t);
 
 cudaError_t preload_fitness64() {
-  cudaError_t e = touch_variant<kPT, 8, false, 1, double, kNW>();
-  if (e == cudaSuccess) e = touch_variant<kPT, 8, true, 1, double, kNW>();
+  cudaError_t e = touch_variant<kPT64, 8, false, 1, double, kNW>();
+  if (e == cudaSuccess) e = touch_variant<kPT64, 8, true, 1, double, kNW>();
   return e;
 }
 

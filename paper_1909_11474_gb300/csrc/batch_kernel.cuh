@@ -23,6 +23,9 @@
 //    the per-(parameter set, configuration) totals and residuals are formed in FP64.
 #pragma once
 
+#include <type_traits>
+
+#include "atom64.cuh"
 #include "common.cuh"
 #include "ctx.hpp"
 
@@ -107,6 +110,18 @@ __device__ __forceinline__ void bond_order(T zeta, const PConsts<T> &K, T &b, T 
 template <typename R>
 struct AtomAcc {
   R U, W[6];
+};
+// What the sums W are to be multiplied with to give the virial (see atom_core_f64).
+template <typename R>
+constexpr R kVirialScale = sizeof(R) == 8 ? R(-2) : R(1);
+// FP64: the parameter set's constants in fixed point (per lane) and the tables of fx64.cuh; nothing in FP32.
+template <typename R>
+struct LaneOrder {};
+template <>
+struct LaneOrder<double> {
+  const FxLane *lane;
+  const FxTables *tab;
+  const double *kc;
 };
 
 // Row stride of the P_ij stage [bond][3][PT] (elements). With 2 or 4 atoms in a warp (PT = 16, 8) the
@@ -420,7 +435,7 @@ __device__ __forceinline__ void atom_forward(const typename Vec4<R>::T *__restri
                                              const typename Vec4<R>::T *__restrict__ sB,
                                              const R *__restrict__ sC, R *__restrict__ stage,
                                              int lb, int lq, int m, bool store, int pl,
-                                             const PConsts<R> &K, AtomAcc<R> &acc) {
+                                             const PConsts<R> &K, const LaneOrder<R> &order, AtomAcc<R> &acc) {
   R ux[M], uy[M], uz[M], r[M], ir2[M], fc[M], fcp[M];
 #pragma unroll
   for (int j = 0; j < M; ++j) {
@@ -466,7 +481,23 @@ __device__ __forceinline__ void atom_forward(const typename Vec4<R>::T *__restri
   }
 
   R U, Px[M], Py[M], Pz[M];
-  if constexpr (sizeof(R) == 4 && !GEN && M % 2 == 0)
+  if constexpr (sizeof(R) == 8) {
+    // FP64: the virial sums come with the core (W += sum u (x) T, scaled by kVirialScale at the end); short lists
+    // of which every bond of the warp is inside R1 (f_C = 1 and f_C' = 0 to the bit) fold the cutoff away
+    bool outer = !EXACT || M > 4;
+    if constexpr (EXACT && M <= 4) {
+#pragma unroll
+      for (int j = 0; j < M; ++j)
+        outer |= __double_as_longlong(fc[j]) != 0x3ff0000000000000ll || (__double_as_longlong(fcp[j]) << 1) != 0;
+      outer = __any_sync(0xffffffffu, outer);
+    }
+    if constexpr (EXACT && M <= 4) {
+      if (!outer)
+        atom_core_f64<M, true, GEN, (M != 4)>(ux, uy, uz, r, ir2, fc, fcp, cs, K, *order.lane, *order.tab, order.kc, U, acc.W, Px, Py, Pz);
+    }
+    if (outer)
+      atom_core_f64<M, false, GEN, true>(ux, uy, uz, r, ir2, fc, fcp, cs, K, *order.lane, *order.tab, order.kc, U, acc.W, Px, Py, Pz);
+  } else if constexpr (!GEN && M % 2 == 0)
     atom_core_x2<M, INNER>(ux, uy, uz, r, ir2, fc, fcp, cs, K, U, Px, Py, Pz);
   else
     atom_core<M, INNER, R, R, GEN>(ux, uy, uz, r, ir2, fc, fcp, cs, K, U, Px, Py, Pz);
@@ -475,7 +506,7 @@ __device__ __forceinline__ void atom_forward(const typename Vec4<R>::T *__restri
 #pragma unroll
   for (int j = 0; j < M; ++j) {
     if (store && (EXACT || j < m)) stage_store<PT, R>(stage, lb + j, pl, Px[j], Py[j], Pz[j]);
-    if (store) {
+    if (sizeof(R) == 4 && store) {
       const R dx = r[j] * ux[j], dy = r[j] * uy[j], dz = r[j] * uz[j];
       acc.W[0] -= dx * Px[j]; acc.W[1] -= dy * Py[j]; acc.W[2] -= dz * Pz[j];
       acc.W[3] -= dx * Py[j]; acc.W[4] -= dy * Pz[j]; acc.W[5] -= dz * Px[j];
@@ -488,11 +519,12 @@ template <int PT, int MMAX, bool EXACT, bool INNER, typename R, bool GEN = false
 __device__ __forceinline__ void atom_forward_dispatch(int Mw, const typename Vec4<R>::T *sA,
                                                       const typename Vec4<R>::T *sB, const R *sC,
                                                       R *stage, int lb, int lq, int m, bool store,
-                                                      int pl, const PConsts<R> &K, AtomAcc<R> &acc) {
+                                                      int pl, const PConsts<R> &K, const LaneOrder<R> &order,
+                                                      AtomAcc<R> &acc) {
 #define TSF_CASE(MM)                                                                          \
   case MM:                                                                                    \
     if constexpr (MMAX >= MM)                                                                 \
-      atom_forward<MM, PT, EXACT, INNER, R, GEN>(sA, sB, sC, stage, lb, lq, m, store, pl, K, acc); \
+      atom_forward<MM, PT, EXACT, INNER, R, GEN>(sA, sB, sC, stage, lb, lq, m, store, pl, K, order, acc); \
     break;
   switch (Mw) {
     TSF_CASE(1) TSF_CASE(2) TSF_CASE(3) TSF_CASE(4) TSF_CASE(5) TSF_CASE(6) TSF_CASE(7) TSF_CASE(8)
@@ -776,6 +808,7 @@ struct TileEnv {
   const double *tgt;               // fitness: the configuration's targets E*, W*_1..6 (shared memory)
   uint8_t mask;
   unsigned rank, ncta;
+  const FxTables *fx;              // FP64: tables of fx64.cuh in shared memory
 };
 
 template <int PTT, int PTW, int MMAX, bool CLUSTER, typename R, int NW, bool GEN, bool FIT>
@@ -813,6 +846,17 @@ __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R>
 #pragma unroll
   for (int k = 0; k < 6; ++k) acc.W[k] = R(0);
 
+  LaneOrder<R> order;
+  std::conditional_t<sizeof(R) == 8, FxLane, int> fxl;
+  if constexpr (sizeof(R) == 8) {
+    order.kc = reinterpret_cast<const double *>(a.consts) + (size_t)(GEN ? 16 : 8) * (active ? p : a.P - 1);
+    order.tab = env.fx;
+    fxl = fx_lane_of<GEN>(order.kc, *env.fx);
+    order.lane = &fxl;
+  } else {
+    (void)fxl;
+  }
+
   // ---- passes 1-2
   for (int base = warp * APW; base < ns; base += NW * APW) {
     const int li = base + slot;
@@ -826,9 +870,9 @@ __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R>
         continue;
       }
       if (sizeof(R) == 4 && at.w == 0)
-        atom_forward_dispatch<PTT, MMAX, true, sizeof(R) == 4, R, GEN>(m, sA, sB, sC, stage, at.x, at.y, m, true, pl, K, acc);
+        atom_forward_dispatch<PTT, MMAX, true, sizeof(R) == 4, R, GEN>(m, sA, sB, sC, stage, at.x, at.y, m, true, pl, K, order, acc);
       else
-        atom_forward_dispatch<PTT, MMAX, true, false, R, GEN>(m, sA, sB, sC, stage, at.x, at.y, m, true, pl, K, acc);
+        atom_forward_dispatch<PTT, MMAX, true, false, R, GEN>(m, sA, sB, sC, stage, at.x, at.y, m, true, pl, K, order, acc);
     } else {
       const int Mw = __reduce_max_sync(0xffffffffu, (unsigned)m);
       const bool uniform = __all_sync(0xffffffffu, m == Mw);
@@ -837,11 +881,11 @@ __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R>
         continue;
       }
       if (uniform && sizeof(R) == 4 && __all_sync(0xffffffffu, at.w == 0))
-        atom_forward_dispatch<PTT, MMAX, true, sizeof(R) == 4, R, GEN>(Mw, sA, sB, sC, stage, at.x, at.y, m, valid, pl, K, acc);
+        atom_forward_dispatch<PTT, MMAX, true, sizeof(R) == 4, R, GEN>(Mw, sA, sB, sC, stage, at.x, at.y, m, valid, pl, K, order, acc);
       else if (uniform)
-        atom_forward_dispatch<PTT, MMAX, true, false, R, GEN>(Mw, sA, sB, sC, stage, at.x, at.y, m, valid, pl, K, acc);
+        atom_forward_dispatch<PTT, MMAX, true, false, R, GEN>(Mw, sA, sB, sC, stage, at.x, at.y, m, valid, pl, K, order, acc);
       else
-        atom_forward_dispatch<PTT, MMAX, false, false, R, GEN>(Mw, sA, sB, sC, stage, at.x, at.y, m, valid, pl, K, acc);
+        atom_forward_dispatch<PTT, MMAX, false, false, R, GEN>(Mw, sA, sB, sC, stage, at.x, at.y, m, valid, pl, K, order, acc);
     }
   }
   if constexpr (CLUSTER) cluster_sync_all(); else __syncthreads();
@@ -849,7 +893,8 @@ __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R>
   // ---- pass 3: F_i = sum_j (P_ij - P_ji)
   R sf = R(0);   // sum |F - F*|^2 over the warp's atoms, or sum |F|^2 without a force target
   // F of atom li in the variants with several atoms in a warp: the own and the reverse rows summed in order,
-  // as in gather_sum
+  // as in gather_sum. Tiles of the kernel's own width find the reverse rows in srev, narrow last tiles (whose
+  // srev holds offsets in the full-width stage) in the bond record
   auto gather_loop = [&](int li, const int4 &at, R (&F)[3]) {
     const int m = at.z, lb = at.x;
     R o[3] = {R(0), R(0), R(0)}, r[3] = {R(0), R(0), R(0)};
@@ -859,10 +904,17 @@ __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R>
       o[0] += x;
       o[1] += y;
       o[2] += z;
-      int packed;  // configuration-local index of the reverse entry in bits 0-15
-      if constexpr (sizeof(R) == 4) packed = __float_as_int((float)sld(&sB[lb + e].w, 14));
-      else packed = (int)sld(&sB[lb + e].w, 14);
-      stage_load<PTT, R>(stage, (packed & 0xffff) + cb0 - B0, pl, x, y, z, 15);
+      if constexpr (CLUSTER) {
+        const unsigned row = (unsigned)sld(reinterpret_cast<const int *>(env.srev) + li * (4 * rev_words<MMAX, true>()) + e, 14);
+        x = ld_cluster(row + pl * sizeof(R), R(0));
+        y = ld_cluster(row + (PTT + pl) * sizeof(R), R(0));
+        z = ld_cluster(row + (2 * PTT + pl) * sizeof(R), R(0));
+      } else {
+        int rb;    // configuration-local index of the reverse entry
+        if constexpr (PTT == PTW) rb = sld(reinterpret_cast<const unsigned short *>(env.srev + li) + e, 14);
+        else rb = __float_as_int((float)sld(&sB[lb + e].w, 14)) & 0xffff;
+        stage_load<PTT, R>(stage, rb + cb0 - B0, pl, x, y, z, 15);
+      }
       r[0] += x;
       r[1] += y;
       r[2] += z;
@@ -945,7 +997,7 @@ __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R>
   R v[kNSum];
   v[0] = acc.U;
 #pragma unroll
-  for (int k = 0; k < 6; ++k) v[1 + k] = acc.W[k];
+  for (int k = 0; k < 6; ++k) v[1 + k] = kVirialScale<R> == R(1) ? acc.W[k] : kVirialScale<R> * acc.W[k];
   v[7] = sf;
 #pragma unroll
   for (int k = 0; k < kNSum; ++k) v[k] = sum_over_atom_slots<PTT>(v[k]);
@@ -1044,10 +1096,14 @@ __global__ void __launch_bounds__(NW * kWarp, MINB) batch_kernel(const BatchPara
   __shared__ double s_fr[kMaxCluster];   // rank 0 of a cluster: the ranks' sums
   __shared__ double s_tgt[7];            // fitness: targets E*, W*_1..6 of the item's configuration
   R *stage = reinterpret_cast<R *>(smem);
-  constexpr int APW = kWarp / PT;
+  __shared__ std::conditional_t<sizeof(R) == 8, FxTables, int> s_fx;
+  const FxTables *fx = nullptr;
+  if constexpr (sizeof(R) == 8) {   // read after the barriers of the first item
+    fx_load_tables(s_fx);
+    fx = &s_fx;
+  }
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int slot = lane / PT, pl = lane % PT;
 
   unsigned rank = 0, ncta = 1;
   if constexpr (CLUSTER) {
@@ -1254,7 +1310,7 @@ __global__ void __launch_bounds__(NW * kWarp, MINB) batch_kernel(const BatchPara
       }
     }
     const TileEnv<R> env = {stage, sA, sB, sC, satom, srev, stF, ns, s0, nat, c, cb0, B0, rec.inv_nat, s_tgt, mask,
-                             rank, ncta};
+                             rank, ncta, fx};
     pdl_wait();   // per-call constants of the preparation kernel (a no-op after the first item)
     // the last tile may hold fewer parameter sets: the FP32 single-CTA variants for up to 4 neighbours
     // run it with more atoms in a warp (tiles of 16 or 8 parameter sets); other variants keep the

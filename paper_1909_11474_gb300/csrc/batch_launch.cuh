@@ -7,13 +7,17 @@
 
 namespace tsf {
 
-constexpr int kPT = 32;   // parameter sets per warp: one atom per warp
+constexpr int kPT = 32;   // parameter sets per warp in FP32: one atom per warp
+// FP64: four atoms x eight parameter sets per warp. The FP64 unit bounds those kernels whatever their loads, so what
+// counts is that no lane works for nothing and that a 64-atom cell's stage leaves the CTA alone on its SM (77 KB
+// instead of 213 KB and a cluster of two): 73 sets take 80 lanes instead of 96, one set 8 instead of 32.
+constexpr int kPT64 = 8;
 
 template <int PTV, int MMAX, bool CLUSTER, int MINB, typename R, int NW, bool GEN, bool FIT>
 inline cudaError_t launch_variant(BatchParams bp, const Bucket &b, bool pdl, cudaStream_t s) {
   auto kern = batch_kernel<PTV, MMAX, CLUSTER, MINB, R, NW, GEN, FIT>;
-  const size_t smem = PTV != kPT ? b.smem16 : NW != kNW ? b.smem12 : b.smem;
-  int &per_sm = b.per_sm[PTV != kPT ? 4 : NW != kNW ? 5 : 2 * (GEN ? 1 : 0) + (FIT ? 1 : 0)];
+  const size_t smem = PTV == 16 ? b.smem16 : NW != kNW ? b.smem12 : b.smem;
+  int &per_sm = b.per_sm[PTV == 16 ? 4 : NW != kNW ? 5 : 2 * (GEN ? 1 : 0) + (FIT ? 1 : 0)];
   constexpr int kThr = NW * kWarp;
   bp.ntiles = (bp.P + PTV - 1) / PTV;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -29,12 +33,26 @@ inline cudaError_t launch_variant(BatchParams bp, const Bucket &b, bool pdl, cud
   }
   const int slots = std::max(1, per_sm * nsm / ncta);
   const int nconf = b.nitems;
-  // work items: whole configurations when they are all alike and fit in one wave of CTAs (the
-  // geometry is then staged once per configuration); otherwise each configuration's tiles are split
-  // into chunks so that about four items per CTA slot balance the dynamically claimed work; the
-  // autotuner's choice for this (P, mode) overrides both
-  int per_conf = 1;
-  if (!(b.uniform && nconf <= slots)) per_conf = std::min(bp.ntiles, std::max(1, (4 * slots + nconf - 1) / nconf));
+  // work items: each configuration's tiles are split into chunks. Ragged configurations: about four items per
+  // CTA slot balance the dynamically claimed work. Alike ones: the chunk with the least time, waves of items x
+  // (tiles + staging), staging an item costing about half a tile (FP32) or a tenth (FP64); fewer items win a tie.
+  // (300 cells on 304 slots stay whole; 100 cells x 2 tiles run as 200 items, 100 cells x 10 FP64 tiles on 152
+  // slots as 1000.) The autotuner's choice for this (P, mode) overrides both
+  int per_conf = std::min(bp.ntiles, std::max(1, (4 * slots + nconf - 1) / nconf));
+  if (b.uniform) {
+    const double stage_cost = sizeof(R) == 8 ? 0.1 : 0.5;
+    double best = 1e300;
+    for (int ct = bp.ntiles; ct >= 1; --ct) {
+      const int nch = (bp.ntiles + ct - 1) / ct;
+      if ((bp.ntiles + nch - 1) / nch != ct) continue;   // the same number of chunks with fewer tiles each comes later
+      const int64_t waves = ((int64_t)nconf * nch + slots - 1) / slots;
+      const double cost = (double)waves * (ct + stage_cost);
+      if (cost < 0.999 * best) {
+        best = cost;
+        per_conf = nch;
+      }
+    }
+  }
   bp.narrow = 1;
   if (b.tune_P == bp.P && b.tune_mode == bp.mode && b.tune_per_conf > 0) {
     per_conf = std::min(bp.ntiles, b.tune_per_conf);
@@ -80,8 +98,8 @@ template <typename R, bool GEN, bool FIT>
 cudaError_t launch_bucket(const BatchParams &bp, const Bucket &b, bool pdl, cudaStream_t s) {
   const bool cl = b.cluster > 1;
   if constexpr (sizeof(R) == 8) {
-    if (!cl) return launch_variant<kPT, 8, false, 1, R, kNW, GEN, FIT>(bp, b, pdl, s);
-    return launch_variant<kPT, 8, true, 1, R, kNW, GEN, FIT>(bp, b, pdl, s);
+    if (!cl) return launch_variant<kPT64, 8, false, 1, R, kNW, GEN, FIT>(bp, b, pdl, s);
+    return launch_variant<kPT64, 8, true, 1, R, kNW, GEN, FIT>(bp, b, pdl, s);
   } else if constexpr (GEN) {
     if (!cl && b.mmax <= 4) return launch_variant<kPT, 4, false, 2, R, kNW, GEN, FIT>(bp, b, pdl, s);
     if (!cl) return launch_variant<kPT, 8, false, 2, R, kNW, GEN, FIT>(bp, b, pdl, s);

@@ -52,7 +52,7 @@ int build_plan(tersoff_ctx *ctx, int precision) {
   Ctx &c = ctx->c;
   tsf::BatchPlan &plan = precision == 64 ? c.plan64 : c.plan32;
   if (plan.precision == precision && !plan.buckets.empty()) return TERSOFF_OK;
-  const int optin = tsf::batch_max_smem_optin();
+  const int optin = tsf::batch_max_smem_optin(precision);
   const size_t soft = std::min<size_t>((size_t)optin, 112 * 1024);  // two CTAs per SM
   struct Key {
     int mmax, cl;
@@ -758,7 +758,7 @@ int tersoff_schedule_info(tersoff_ctx *ctx, int32_t precision, int32_t bucket, i
   info[1] = b.cluster;
   info[2] = b.nitems;
   info[3] = tuned ? b.tune_P : 0;
-  info[4] = tuned ? b.tune_pt : 32;
+  info[4] = tuned && b.tune_pt != 32 ? b.tune_pt : tsf::batch_param_tile(precision);
   info[5] = tuned ? b.tune_per_conf : 0;
   info[6] = tuned ? b.tune_narrow : 1;
   info[7] = tuned ? b.tune_nw : 8;

@@ -315,8 +315,8 @@ cudaError_t launch_plain(const Ctx &ctx, const double *params, int P, double *E,
 size_t batch_smem_bytes_pt(int precision, int nb, int nq, int nat, int ncta);   // ncta = cluster size
 size_t batch_smem_bytes_pt16(int nb, int nq, int nat);   // FP32 single-CTA, 16 parameter sets per tile
 size_t batch_smem_bytes_nw12(int nb, int nq, int nat);   // FP32 single-CTA, 12 warps per CTA
-int batch_param_tile();
-int batch_max_smem_optin();
+int batch_param_tile(int precision);
+int batch_max_smem_optin(int precision);
 
 }  // namespace tsf
 

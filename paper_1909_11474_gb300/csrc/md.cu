@@ -632,7 +632,7 @@ __device__ __forceinline__ void md_atom(const R (&ux)[M], const R (&uy)[M], cons
 // Fixed-order block sum of n values per quantity, src[k * stride + q] (q < n, k < K): a strided sum
 // per thread (loads in flight together), a butterfly over each warp's lanes, then the warps in order
 // (through `red`, [warps][>= K]); thread k < K returns quantity k.
-template <int K>
+template <int K, int TH>
 __device__ __forceinline__ double md_block_sum(const double *src, size_t stride, int n, double (*red)[7]) {
   const int tid = threadIdx.x;
   double acc[K];
@@ -640,7 +640,7 @@ __device__ __forceinline__ double md_block_sum(const double *src, size_t stride,
   for (int k = 0; k < K; ++k) {
     acc[k] = 0.0;
 #pragma unroll 4
-    for (int q = tid; q < n; q += kMdThreads) acc[k] += __ldcg(&src[k * stride + q]);
+    for (int q = tid; q < n; q += TH) acc[k] += __ldcg(&src[k * stride + q]);
     for (int off = 16; off > 0; off >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], off);
   }
   __syncthreads();                                 // earlier readers of red are done
@@ -650,17 +650,17 @@ __device__ __forceinline__ double md_block_sum(const double *src, size_t stride,
   __syncthreads();
   double s = 0.0;
   if (tid < K)
-    for (int w = 0; w < kMdThreads / 32; ++w) s += red[w][tid];
+    for (int w = 0; w < TH / 32; ++w) s += red[w][tid];
   return s;
 }
 
-// Deterministic in-kernel sum of per-block partials [K][nblk] (FP64; blocks of kMdThreads threads):
+// Deterministic in-kernel sum of per-block partials [K][nblk] (FP64; blocks of TH threads):
 // the last block of each group of kMdGroup blocks to finish sums its group into [K][ngroups], and
 // the last group to finish sums the groups, both in a fixed order; quantity 0 goes to *out0 and
 // quantity k >= 1 to out_rest[k - 1]. The group sums follow the partials; the counters [ngroups + 1]
 // are zeroed before the launch. The threads that wrote the block's partials have fenced before the call.
 constexpr int kMdGroup = 64;
-template <int K>
+template <int K, int TH>
 __device__ __forceinline__ void md_grouped_sum(double *partial, unsigned *counter, int nblk, int b, double *out0,
                                                double *out_rest, double (*red)[7]) {
   __shared__ int s_last;
@@ -672,7 +672,7 @@ __device__ __forceinline__ void md_grouped_sum(double *partial, unsigned *counte
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  const double t = md_block_sum<K>(partial + g0, (size_t)nblk, gn, red);
+  const double t = md_block_sum<K, TH>(partial + g0, (size_t)nblk, gn, red);
   if (tid < K) {
     gpart[(size_t)tid * ngroups + g] = t;
     __threadfence();
@@ -682,7 +682,7 @@ __device__ __forceinline__ void md_grouped_sum(double *partial, unsigned *counte
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  const double u = md_block_sum<K>(gpart, (size_t)ngroups, ngroups, red);
+  const double u = md_block_sum<K, TH>(gpart, (size_t)ngroups, ngroups, red);
   if (tid == 0) *out0 = u;
   else if (tid < K) out_rest[tid - 1] = u;
 }
@@ -739,7 +739,8 @@ __device__ __forceinline__ void md_force_atom(int N, int M, int i, int m, const 
                                               const unsigned *__restrict__ keys, const int *__restrict__ cnt,
                                               const int *__restrict__ nbr, const char4 *__restrict__ shift,
                                               float4 xi, typename Vec4<R>::T *__restrict__ Prev,
-                                              unsigned *status, R &U, R (&Wv)[6], R (&Fo)[3]) {
+                                              const LaneOrder<R> &order, unsigned *status, R &U, R (&Wv)[6],
+                                              R (&Fo)[3]) {
   using R4 = typename Vec4<R>::T;
   constexpr int M_ = Mw;
   R ux[M_], uy[M_], uz[M_], r[M_], ir[M_], fc[M_], fcp[M_];
@@ -761,15 +762,28 @@ __device__ __forceinline__ void md_force_atom(int N, int M, int i, int m, const 
       } else {
         const int j = nbr[(size_t)e * N + i];
         const char4 n = shift[(size_t)e * N + i];
-        const ExactPair p = exact_pair(pos[3 * j], pos[3 * j + 1], pos[3 * j + 2], pos[3 * i], pos[3 * i + 1],
-                                       pos[3 * i + 2], G.H, n.x, n.y, n.z);
-        dx = p.dx;
-        dy = p.dy;
-        dz = p.dz;
+        if ((n.x | n.y | n.z) == 0) {   // no image shift (all but the atoms near a face): t is exactly zero
+          dx = pos[3 * j] - pos[3 * i];
+          dy = pos[3 * j + 1] - pos[3 * i + 1];
+          dz = pos[3 * j + 2] - pos[3 * i + 2];
+        } else {
+          const ExactPair p = exact_pair(pos[3 * j], pos[3 * j + 1], pos[3 * j + 2], pos[3 * i], pos[3 * i + 1],
+                                         pos[3 * i + 2], G.H, n.x, n.y, n.z);
+          dx = p.dx;
+          dy = p.dy;
+          dz = p.dz;
+        }
       }
-      const R rr = sqrt(dx * dx + dy * dy + dz * dz);
+      R rr;
+      if constexpr (sizeof(R) == 4) {
+        rr = sqrt(dx * dx + dy * dy + dz * dz);
+        ir[e] = R(1) / rr;
+      } else {
+        const R r2 = dx * dx + dy * dy + dz * dz;
+        ir[e] = rsqrt64(r2);
+        rr = __double_as_longlong(r2) == 0 ? R(0) : r2 * ir[e];   // coincident atoms: r = 0, as the square root gives
+      }
       r[e] = rr;
-      ir[e] = R(1) / rr;
       ux[e] = dx * ir[e];
       uy[e] = dy * ir[e];
       uz[e] = dz * ir[e];
@@ -782,7 +796,7 @@ __device__ __forceinline__ void md_force_atom(int N, int M, int i, int m, const 
           fcp[e] = G.fcp_kf * sinpif(w);
         }
       } else {
-        if (rr <= G.R1) {
+        if (__double_as_longlong(rr) <= __double_as_longlong(G.R1)) {   // both positive: ordered as integers
           fc[e] = 1.0;
         } else if (rr < G.R2) {
           const double w = (rr - G.R1) * G.inv_w;
@@ -793,7 +807,32 @@ __device__ __forceinline__ void md_force_atom(int N, int M, int i, int m, const 
     }
   }
   R Px[M_], Py[M_], Pz[M_];
-  md_atom<M_, R>(ux, uy, uz, r, ir, fc, fcp, K, U, Wv, Px, Py, Pz);
+  if constexpr (sizeof(R) == 4) {
+    md_atom<M_, R>(ux, uy, uz, r, ir, fc, fcp, K, U, Wv, Px, Py, Pz);
+  } else {
+    // the core of the batched FP64 kernels: W comes as sum u (x) T, to be scaled by kVirialScale; four bonds, all
+    // inside R1, in every lane fold the cutoff away
+    constexpr int NP = M_ * (M_ - 1) / 2;
+    R cs[NP > 0 ? NP : 1], ir2[M_], Ui;
+    bool outer = M_ != 4;
+#pragma unroll
+    for (int j = 0; j < M_; ++j) {
+      ir2[j] = j < m ? scale2(ir[j], 1) : R(0);
+      outer |= __double_as_longlong(fc[j]) != 0x3ff0000000000000ll || (__double_as_longlong(fcp[j]) << 1) != 0;
+    }
+    int q = 0;
+#pragma unroll
+    for (int j = 0; j < M_; ++j)
+#pragma unroll
+      for (int k = j + 1; k < M_; ++k) cs[q++] = ux[j] * ux[k] + uy[j] * uy[k] + uz[j] * uz[k];
+    if (M_ == 4 && !__any_sync(0xffffffffu, outer))
+      atom_core_f64<M_, true, false, (M_ != 4)>(ux, uy, uz, r, ir2, fc, fcp, cs, K, *order.lane, *order.tab, order.kc, Ui, Wv,
+                                                Px, Py, Pz);
+    else
+      atom_core_f64<M_, false, false, true>(ux, uy, uz, r, ir2, fc, fcp, cs, K, *order.lane, *order.tab, order.kc, Ui, Wv, Px,
+                                            Py, Pz);
+    U += R(0.5) * Ui;
+  }
 #pragma unroll
   for (int e = 0; e < M_; ++e)
     if (e < m) {
@@ -801,12 +840,18 @@ __device__ __forceinline__ void md_force_atom(int N, int M, int i, int m, const 
       Fo[1] += Py[e];
       Fo[2] += Pz[e];
       if (rs[e] >= 0) {
-        R4 v;
-        v.x = Px[e];
-        v.y = Py[e];
-        v.z = Pz[e];
-        v.w = R(0);
-        Prev[rs[e]] = v;
+        if constexpr (sizeof(R) == 4) {
+          R4 v;
+          v.x = Px[e];
+          v.y = Py[e];
+          v.z = Pz[e];
+          v.w = R(0);
+          Prev[rs[e]] = v;
+        } else {   // two 16-byte stores: as one 32-byte store the y and z of the called functions came out wrong
+          double2 *o = reinterpret_cast<double2 *>(Prev + rs[e]);
+          o[0] = make_double2(Px[e], Py[e]);
+          o[1] = make_double2(Pz[e], 0.0);
+        }
       }
     }
 }
@@ -823,26 +868,43 @@ __device__ __noinline__ MdSums<R> md_force_atom_long(int N, int M, int i, int m,
                                                      const float4 *__restrict__ x4, const unsigned *__restrict__ keys,
                                                      const int *__restrict__ cnt, const int *__restrict__ nbr,
                                                      const char4 *__restrict__ shift, float4 xi,
-                                                     typename Vec4<R>::T *__restrict__ Prev, unsigned *status) {
+                                                     typename Vec4<R>::T *__restrict__ Prev,
+                                                     const LaneOrder<R> &order, unsigned *status) {
   MdSums<R> o;
   o.U = R(0);
 #pragma unroll
   for (int k = 0; k < 6; ++k) o.W[k] = R(0);
   o.F[0] = o.F[1] = o.F[2] = R(0);
-  md_force_atom<Mw, R>(N, M, i, m, G, K, pos, x4, keys, cnt, nbr, shift, xi, Prev, status, o.U, o.W, o.F);
+  md_force_atom<Mw, R>(N, M, i, m, G, K, pos, x4, keys, cnt, nbr, shift, xi, Prev, order, status, o.U, o.W, o.F);
   return o;
 }
 
-template <typename R>
-__global__ void __launch_bounds__(kMdThreads, sizeof(R) == 4 ? 8 : 1) md_force_kernel(
-    int N, int M, const MdGeom G, const PConsts<R> K, const double *__restrict__ pos,
+// TH threads a block: FP32 128. FP64, bound by the FP64 unit of the SMs that have a block (about 300 of its
+// instructions an atom), 32 for small systems, so that 4,096 atoms reach 128 SMs instead of 32, and 128 for large ones,
+// where the table copies of more blocks would only cost.
+template <typename R, int TH>
+__global__ void __launch_bounds__(TH, sizeof(R) == 4 ? 8 : 1) md_force_kernel(
+    int N, int M, const __grid_constant__ MdGeom G, const __grid_constant__ PConsts<R> K, const double *__restrict__ pos,
     const float4 *__restrict__ x4, const unsigned *__restrict__ keys, const int *__restrict__ cnt,
     const int *__restrict__ nbr, const char4 *__restrict__ shift, typename Vec4<R>::T *__restrict__ Fown,
     typename Vec4<R>::T *__restrict__ Prev, double *__restrict__ partial, unsigned *counters, double *__restrict__ E,
     double *__restrict__ W, unsigned *status) {
-  __shared__ double red[kMdThreads / 32][7];
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ double red[TH / 32][7];
+  __shared__ std::conditional_t<sizeof(R) == 8, FxTables, int> s_fx;
+  const int i = blockIdx.x * TH + threadIdx.x;
   const bool valid = i < N;
+  LaneOrder<R> order;
+  std::conditional_t<sizeof(R) == 8, FxLane, int> fxl;
+  if constexpr (sizeof(R) == 8) {
+    fx_load_tables(s_fx);
+    __syncthreads();
+    order.kc = &K.D0;                              // the first eight constants are laid out as prep_kernel's
+    order.tab = &s_fx;
+    fxl = fx_lane_of<false>(order.kc, s_fx);
+    order.lane = &fxl;
+  } else {
+    (void)fxl;
+  }
   int m = valid ? min(cnt[i], M) : 0;   // a truncated list (count > M) is flagged; its row holds M entries
   if (m > kMdMaxM) {
     set_status(status, TERSOFF_STATUS_MANY_NBRS);
@@ -856,10 +918,10 @@ __global__ void __launch_bounds__(kMdThreads, sizeof(R) == 4 ? 8 : 1) md_force_k
   const int Mw = __reduce_max_sync(0xffffffffu, (unsigned)m);
   switch (Mw) {
 #define TSF_MDCASE(MM) \
-    case MM: md_force_atom<MM, R>(N, M, i, m, G, K, pos, x4, keys, cnt, nbr, shift, xi, Prev, status, U, Wv, Fo); break;
+    case MM: md_force_atom<MM, R>(N, M, i, m, G, K, pos, x4, keys, cnt, nbr, shift, xi, Prev, order, status, U, Wv, Fo); break;
 #define TSF_MDLONG(MM)                                                                      \
     case MM: {                                                                              \
-      const MdSums<R> o = md_force_atom_long<MM, R>(N, M, i, m, G, K, pos, x4, keys, cnt, nbr, shift, xi, Prev, status); \
+      const MdSums<R> o = md_force_atom_long<MM, R>(N, M, i, m, G, K, pos, x4, keys, cnt, nbr, shift, xi, Prev, order, status); \
       U = o.U;                                                                              \
       for (int k = 0; k < 6; ++k) Wv[k] = o.W[k];                                           \
       for (int k = 0; k < 3; ++k) Fo[k] = o.F[k];                                           \
@@ -881,6 +943,9 @@ __global__ void __launch_bounds__(kMdThreads, sizeof(R) == 4 ? 8 : 1) md_force_k
   }
   // per-warp sums in R, per-block FP64 partial sums of U and W, stored [7][blocks]
   R v[7] = {U, Wv[0], Wv[1], Wv[2], Wv[3], Wv[4], Wv[5]};
+  if constexpr (kVirialScale<R> != R(1))
+#pragma unroll
+    for (int k = 1; k < 7; ++k) v[k] *= kVirialScale<R>;
 #pragma unroll
   for (int k = 0; k < 7; ++k)
     for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], off);
@@ -892,11 +957,11 @@ __global__ void __launch_bounds__(kMdThreads, sizeof(R) == 4 ? 8 : 1) md_force_k
   const int nblk = gridDim.x, b = blockIdx.x, tid = threadIdx.x;
   if (tid < 7) {
     double s = 0.0;
-    for (int w = 0; w < kMdThreads / 32; ++w) s += red[w][tid];
+    for (int w = 0; w < TH / 32; ++w) s += red[w][tid];
     partial[(size_t)tid * nblk + b] = s;
     __threadfence();                               // the partial before this block's count
   }
-  md_grouped_sum<7>(partial, counters, nblk, b, E, W, red);
+  md_grouped_sum<7, TH>(partial, counters, nblk, b, E, W, red);
 }
 
 // F_i = sum_e P_ij - sum_e P_ji over atom i's entries e = (j, n): the first sum from Fown (the force
@@ -992,13 +1057,15 @@ int md_force(Ctx &c, int N, const double *pos, const double *boxh, const double 
     return TERSOFF_E_ARG;
   }
   const int nblk = (N + kMdThreads - 1) / kMdThreads;
-  const int ngroups = (nblk + kMdGroup - 1) / kMdGroup;
+  const bool small64 = precision == 64 && N <= 8 * 32 * c.nsm;   // one warp a block fills no more than an SM's eight
+  const int fblk = small64 ? (N + 31) / 32 : nblk;               // blocks of the force kernel
+  const int ngroups = (fblk + kMdGroup - 1) / kMdGroup;
   const size_t rs = precision == 64 ? 8 : 4;
   if (c.md_cellcnt.ensure((ncells + ngroups + 1) * sizeof(int)) || c.md_cells.ensure(ncells * kMdCap * sizeof(float4)) ||
       c.md_pos.ensure((size_t)N * (sizeof(float4) + sizeof(int4))) || c.md_cnt.ensure((size_t)N * sizeof(int)) ||
       c.md_nbr.ensure((size_t)N * M * sizeof(int)) || c.md_shift.ensure((size_t)N * M * sizeof(char4)) ||
       c.md_keys.ensure((size_t)N * M * sizeof(unsigned)) || c.md_Pij.ensure((size_t)N * (kMdMaxM + 1) * 4 * rs) ||
-      c.md_red.ensure(md_sum_bytes(7, nblk))) {
+      c.md_red.ensure(md_sum_bytes(7, fblk))) {
     err = "device allocation failed";
     return TERSOFF_E_CUDA;
   }
@@ -1022,15 +1089,15 @@ int md_force(Ctx &c, int N, const double *pos, const double *boxh, const double 
   if (precision == 64) {
     PConsts<double> K{D0, -al * log2e, r0, -0.5 * al, be, h, n, -0.5 / n};
     dvec4 *Fown = c.md_Pij.as<dvec4>(), *Prev = Fown + N;
-    md_force_kernel<double><<<nblk, kMdThreads, 0, s>>>(N, M, G, K, pos, x4, keys, cnt, c.md_nbr.as<int>(),
-                                                        c.md_shift.as<char4>(), Fown, Prev, c.md_red.as<double>(), sum_counters,
-                                                        E, W, st);
+    auto force = small64 ? md_force_kernel<double, 32> : md_force_kernel<double, kMdThreads>;
+    force<<<fblk, small64 ? 32 : kMdThreads, 0, s>>>(N, M, G, K, pos, x4, keys, cnt, c.md_nbr.as<int>(), c.md_shift.as<char4>(),
+                                                     Fown, Prev, c.md_red.as<double>(), sum_counters, E, W, st);
     md_gather_kernel<double><<<nblk, kMdThreads, 0, s>>>(N, M, cnt, Fown, Prev, reinterpret_cast<double *>(F));
   } else {
     PConsts<float> K{(float)D0, (float)(-al * log2e), (float)r0, (float)(-0.5 * al), (float)be, (float)h,
                      (float)n, (float)(-0.5 / n)};
     float4 *Fown = c.md_Pij.as<float4>(), *Prev = Fown + N;
-    md_force_kernel<float><<<nblk, kMdThreads, 0, s>>>(N, M, G, K, pos, x4, keys, cnt, c.md_nbr.as<int>(),
+    md_force_kernel<float, kMdThreads><<<nblk, kMdThreads, 0, s>>>(N, M, G, K, pos, x4, keys, cnt, c.md_nbr.as<int>(),
                                                        c.md_shift.as<char4>(), Fown, Prev, c.md_red.as<double>(), sum_counters,
                                                        E, W, st);
     md_gather_kernel<float><<<nblk, kMdThreads, 0, s>>>(N, M, cnt, Fown, Prev, reinterpret_cast<float *>(F));
@@ -1101,7 +1168,7 @@ __global__ void __launch_bounds__(kMdThreads) md_kick_kernel(int N, double *__re
     partial[blockIdx.x] = s;
     __threadfence();
   }
-  md_grouped_sum<1>(partial, counters, gridDim.x, blockIdx.x, Ekin, nullptr, red);
+  md_grouped_sum<1, kMdThreads>(partial, counters, gridDim.x, blockIdx.x, Ekin, nullptr, red);
 }
 
 int md_nve(Ctx &c, int N, double *pos, double *vel, const double *mass, const double *boxh, const double *x,

@@ -1,0 +1,89 @@
+"""The fixed-point 2^x / log2 functions of csrc/fx64.cuh, compiled for the host (their arithmetic is the device's, bit
+for bit): accuracy against extended precision over the potential's ranges and far beyond, and what they refuse."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1909_11474_gb300", "csrc")
+
+SRC = r"""
+#include <cmath>
+#include <cstdint>
+#include <cstdio>
+#include <cstring>
+#include <random>
+#define __host__
+#define __device__
+#define __forceinline__ inline
+#include "fx64.cuh"
+#include "fx64_tables.inc"
+using namespace tsf;
+typedef long double Q;
+int main() {
+  static FxTables t;
+  for (int j = 0; j < 256; ++j) { t.exp2[j] = kFxExp2[j]; t.log_inv[j] = kFxLogInv[j]; t.inv[j] = kFxInv[j]; }
+  std::mt19937_64 g(7);
+  std::uniform_real_distribution<double> U(0, 1);
+  double worst[2][3] = {{0, 0, 0}, {0, 0, 0}};
+  int refused[2] = {0, 0};
+  for (int i = 0; i < 400000; ++i) {
+    const int wide = i & 1;
+    double D0 = 3.2 * (0.7 + 0.6 * U(g)), al = 1.43 * (0.7 + 0.6 * U(g)), r0 = 2.238 * (0.7 + 0.6 * U(g));
+    double be = 0.28 * (0.7 + 0.6 * U(g)), n = 0.6 * (0.7 + 0.6 * U(g)), r = 1.9 + 1.3 * U(g), S = 0.001 + 2 * U(g);
+    if (wide) {
+      D0 = std::exp((U(g) - 0.5) * 60); al = 4 * U(g); be = std::exp((U(g) - 0.5) * 40); n = 0.02 + 3.9 * U(g);
+      r = 0.2 + 6 * U(g); S = std::exp((U(g) - 0.7) * 60);
+    }
+    if (i % 17 == 0) S = 0;
+    if (i % 19 == 0) S = std::ldexp(1.0 + (i % 5 - 2) * 0x1p-52, i % 7 - 3);   // beside powers of two
+    if (i % 23 == 0) r = r0;
+    const double k = -al * 1.4426950408889634, in = -0.5 / n;
+    double fR, bh, cc;
+    if (!fx_bond(r, S, fx_lane(r0, k, 2 * k, D0, D0, be, n, in, t), t, fR, bh, cc)) { ++refused[wide]; continue; }
+    const Q x = std::exp2((Q)k * ((Q)r - (Q)r0)), hA = D0 * x;
+    Q z = (Q)be * (Q)S;
+    if (z < (Q)1e-30) z = 1e-30;
+    const Q zn = std::pow(z, (Q)n), b = std::pow(1 + zn, (Q)in);
+    const Q ref[3] = {hA * x, b * hA, (Q)be * b * hA * zn / (2 * z * (1 + zn))};
+    const double got[3] = {fR, bh, cc};
+    for (int q = 0; q < 3; ++q) {
+      const double e = (double)std::fabs((got[q] - ref[q]) / ref[q]);
+      if (!(e <= worst[wide][q])) worst[wide][q] = e;
+    }
+  }
+  const double inf = INFINITY, nan = NAN;
+  double a, b, c;
+  const FxLane ok = fx_lane(2.2, -2.0, -4.0, 3.2, 3.2, 0.28, 0.6, -0.5 / 0.6, t);
+  int bad = !ok.ok;
+  for (double r : {16.0, 1e300, inf, nan, -inf}) bad += fx_bond(r, 1.0, ok, t, a, b, c);
+  for (double S : {inf, nan, 1e80}) bad += fx_bond(2.3, S, ok, t, a, b, c);
+  for (double v : {0.0, -1.0, inf, nan, 1e-70, 1e70, 5e-324}) bad += fx_lane(2.2, -2, -4, v, 3.2, 0.28, 0.6, -0.5 / 0.6, t).ok;
+  for (double v : {0.0, -1.0, inf, nan}) bad += fx_lane(2.2, -2, -4, 3.2, 3.2, v, 0.6, -0.5 / 0.6, t).ok;
+  for (double v : {0.0, -0.6, 4.0, 0.015, inf, nan}) bad += fx_lane(2.2, -2, -4, 3.2, 3.2, 0.28, v, -0.5 / v, t).ok;
+  for (double v : {16.0, inf, nan}) bad += fx_lane(v, -2, -4, 3.2, 3.2, 0.28, 0.6, -0.5 / 0.6, t).ok + fx_lane(2.2, v, -4, 3.2, 3.2, 0.28, 0.6, -0.5 / 0.6, t).ok;
+  std::printf("%.17g %.17g %.17g %.17g %.17g %.17g %d %d %d\n", worst[0][0], worst[0][1], worst[0][2], worst[1][0],
+              worst[1][1], worst[1][2], refused[0], refused[1], bad);
+}
+"""
+
+
+def test_fixed_point_bond_functions(tmp_path):
+    """Within the potential's ranges every value is within 1.5 x 2^-52 relative (2^-53 of rounding, the rest
+    the fixed-point errors stated in fx64.cuh) plus, far beyond them, the 2^-54 absolute error of an exponent times the
+    largest factor it meets (1/(2n) <= 25: 2^-54 ln2 25 < 1e-15). Nothing in range is refused; every argument outside
+    the ranges is."""
+    cxx = shutil.which("g++")
+    if cxx is None:
+        pytest.skip("no g++")
+    src = tmp_path / "fx.cpp"
+    src.write_text(SRC)
+    exe = tmp_path / "fx"
+    subprocess.run([cxx, "-O2", "-std=c++17", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    v = subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split()
+    worst, (refused, refused_wide, bad) = [float(x) for x in v[:6]], [int(x) for x in v[6:]]
+    assert max(worst[:3]) <= 1.5 * 2.0 ** -52, worst
+    assert max(worst[3:]) <= 1.5e-15, worst
+    assert refused == 0 and bad == 0
+    assert refused_wide < 0.05 * 200000

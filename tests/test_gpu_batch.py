@@ -390,3 +390,44 @@ def test_cluster_gather_on_disordered_cells(precision, reps, vac, sigma):
     assert energy_rel_err(E.cpu().numpy(), Er, ES).max() < tol["E"]
     assert virial_rel_err(W.cpu().numpy(), Wr, WS).max() < tol["W"]
     assert force_err(F.cpu().double().numpy(), Fr, FS) < tol["F"]
+
+
+@pytest.mark.parametrize("form", [0, 1])
+@pytest.mark.parametrize("P", [1, 7, 8, 9, 17])
+def test_fp64_tiles_and_parameter_ranges(P, form):
+    """The FP64 kernel's tiles of eight sets, full and partly filled, over ragged cells (several atoms of different
+    list lengths in a warp; lone atoms and dimers), with parameter sets inside and outside the ranges of its
+    fixed-point functions (n beyond [1/64, 4), prefactors that are negative, tiny or huge, r0 beyond 16): E, F and W
+    of every set equal those of the set evaluated alone, and for the minimal form those of the plain FP64 path (but for
+    where zeta <= 0, the dimer and a negative beta, which the batched kernels clamp to 1e-30 and the plain path takes
+    as b = 1, b' = 0)."""
+    from paper_1909_11474_gb300 import binding
+    rng = np.random.default_rng(17)
+    parts = [(np.array([[0.5, 0.5, 0.5]]), np.eye(3) * 9.0), (np.array([[0.0, 0, 0], [2.3, 0.2, 0]]), np.eye(3) * 12.0)]
+    for reps, sigma, vac in (((1, 1, 1), 0.1, 1), ((2, 2, 2), 0.25, 2), ((2, 3, 2), 0.2, 5)):
+        pos, box = I.diamond_supercell(reps)
+        pos = pos[np.sort(rng.choice(len(pos), len(pos) - vac, replace=False))]
+        parts.append((pos + rng.normal(0, sigma, pos.shape), box))
+    cs = I.pack_configs(*zip(*parts))
+    x0 = I.TABLE2_PARAMS if form == 0 else np.array([3.2, 1.45, 2.25, 1.9, 0.65, -0.6, 0.06, 20.0, 3.0])
+    x = x0[None, :] * (1 + 0.1 * rng.uniform(-1, 1, size=(17, len(x0))))
+    iB = 3 if form == 0 else 6
+    for k, (q, v) in enumerate([(4, 5.0), (4, 0.01), (0, -1.5), (iB, -0.2), (0, 1e-70), (0, 1e80), (2, 17.0), (1, 20.0),
+                                (iB, 1e-65)]):
+        x[(2 * k + 3) % 17, q] = v
+    x[:P] = np.roll(x, -3, axis=0)[:P]
+    ctx = binding.Context(0)
+    ctx.set_form(form)
+    p, b = to_device(cs)
+    ctx.build_neighbors(cs.atom_off, p, b, 2.8, 3.2, 16)
+    xt = torch.tensor(x[:P].copy(), device="cuda")
+    E, F, W = ctx.eval(xt, precision=64)
+    for k in range(P):
+        E1, F1, W1 = ctx.eval(xt[k:k + 1].contiguous(), precision=64)
+        assert torch.equal(E1[0], E[k]) and torch.equal(F1[0], F[k]) and torch.equal(W1[0], W[k])
+    if form == 0:
+        Ep, Fp, Wp = ctx.eval_plain(xt)
+        for got, ref in ((E[:, 2:], Ep[:, 2:]), (F[:, 3:], Fp[:, 3:]), (W[:, 2:], Wp[:, 2:])):
+            for k in np.flatnonzero(x[:P, 3] > 0):
+                assert (got[k] - ref[k]).abs().max() <= 1e-10 * ref[k].abs().max(), (k, x[k])
+    assert ctx.get_status() == 0
