@@ -10,17 +10,18 @@
 #include "common.cuh"
 #include "ctx.hpp"
 #include "fx64.cuh"
-#include "fx64_tables.inc"
 
 namespace tsf {
 
+#include "fx64_tables.inc"
+
 // Fills a kernel's table copy in shared memory (all threads; the caller synchronises).
 __device__ __forceinline__ void fx_load_tables(FxTables &t) {
-  for (int k = threadIdx.x; k < 256; k += blockDim.x) {
-    t.exp2[k] = kFxExp2[k];
-    t.log_inv[k] = kFxLogInv[k];
-    t.inv[k] = kFxInv[k];
-  }
+  constexpr int n = sizeof(FxTables) / sizeof(uint4);
+  const uint4 *src = reinterpret_cast<const uint4 *>(&kFxTables);
+  uint4 *dst = reinterpret_cast<uint4 *>(&t);
+#pragma unroll 10
+  for (int k = threadIdx.x; k < n; k += blockDim.x) dst[k] = src[k];   // one warp: ten loads in flight
 }
 
 // f_R, b f_A / 2 and the coefficient cc of fx_bond.

@@ -34,7 +34,7 @@
 namespace tsf {
 
 // Tables in the caller's memory (shared memory in the kernels; filled from fx64_tables.inc).
-struct FxTables {
+struct alignas(16) FxTables {
   unsigned long long exp2[256];     // 2^(j/256), 63 fraction bits
   unsigned long long log_inv[256];  // -log2(c_j), 62 fraction bits
   unsigned inv[256];                // c_j, 11 fraction bits

@@ -18,12 +18,11 @@ SRC = r"""
 #define __device__
 #define __forceinline__ inline
 #include "fx64.cuh"
-#include "fx64_tables.inc"
 using namespace tsf;
+#include "fx64_tables.inc"
 typedef long double Q;
 int main() {
-  static FxTables t;
-  for (int j = 0; j < 256; ++j) { t.exp2[j] = kFxExp2[j]; t.log_inv[j] = kFxLogInv[j]; t.inv[j] = kFxInv[j]; }
+  const FxTables &t = kFxTables;
   std::mt19937_64 g(7);
   std::uniform_real_distribution<double> U(0, 1);
   double worst[2][3] = {{0, 0, 0}, {0, 0, 0}};

@@ -174,3 +174,26 @@ def test_md_nonfinite_atom_is_flagged_and_left_out(ctx):
         assert np.array_equal(nbr[i, :cnt[i]], idx[nl["j"][e]])
         assert np.array_equal(shift[i, :cnt[i]], nl["n"][e])
     _md(ctx, pos, box, I.TABLE2_PARAMS, 32)      # the next call on finite positions is clean
+
+
+@pytest.mark.parametrize("precision,tiles", [(64, (1, 1, 1)), (64, (4, 3, 3)), (64, (4, 4, 3)), (32, (2, 3, 1)),
+                                             (32, (6, 5, 5)), (32, (7, 5, 5))])
+@pytest.mark.parametrize("sigma,strain", [(0.1, 0.0), (0.24, 0.04)])
+def test_md_tiled_cell_repeats_its_base(ctx, precision, tiles, sigma, strain):
+    """A cell tiled from copies of a disordered (and sheared) base cell has n times its energy and virial and the
+    base's forces on every copy. The tilings straddle the sizes at which the energy and virial sums take a second level
+    (256 blocks: 8,192 atoms in FP64, 32,768 in FP32), leave the bricks of the search and the last blocks partly
+    filled, and hold lists of up to 8 bonds in warps of four lanes an atom (FP64) and of a thread an atom (FP32)."""
+    pos, box = _cell((3, 3, 3), sigma, strain, 11, False)
+    params = I.TABLE2_PARAMS
+    r = oracle.evaluate(pos, box, params)
+    k = np.stack(np.meshgrid(*(np.arange(t) for t in tiles), indexing="ij"), -1).reshape(-1, 1, 3)
+    n = len(k)
+    rng = np.random.default_rng(3)
+    order = rng.permutation(n * len(pos))                      # atoms in no spatial order
+    big = (pos[None] + k @ box).reshape(-1, 3)[order]
+    E, F, W = _md(ctx, np.ascontiguousarray(big), box * np.asarray(tiles)[:, None], params, precision)
+    tol = TOL32 if precision == 32 else TOL64
+    assert energy_rel_err(np.array([E]), np.array([n * r["E"]]), np.array([n * r["E_scale"]])).max() < tol["E"]
+    assert virial_rel_err(W[None], n * r["W"][None], np.array([n * r["W_scale"]])).max() < tol["W"]
+    assert force_err(F, np.tile(r["F"], (n, 1))[order], np.tile(r["F_scale"], n)[order]) < tol["F"]
