@@ -254,17 +254,29 @@ __global__ void __launch_bounds__(kFinWarps * 32) fitness_finalize_kernel(
       v[q] += pp[(size_t)c * kResidualTerms + q];
       v[3 + q] += dpart[3 * c + q];
     }
+  // sums over the warp, an xor tree for each quantity: with offset 16, 8 and 4 each half of the lanes keeps half of the
+  // quantities, so that 9 FP64 additions do it (30 with every lane adding every quantity)
+  double h[4];
 #pragma unroll
-  for (int k = 0; k < 6; ++k)
-    for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], off);
-  if (lane == 0)
+  for (int k = 0; k < 4; ++k) {
+    const double up = k < 2 ? v[4 + k] : 0.0, keep = (lane & 16) ? up : v[k], give = (lane & 16) ? v[k] : up;
+    h[k] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+  }
 #pragma unroll
-    for (int k = 0; k < 6; ++k) s_red[warp][k] = v[k];
+  for (int k = 0; k < 2; ++k) {
+    const double keep = (lane & 8) ? h[k + 2] : h[k], give = (lane & 8) ? h[k] : h[k + 2];
+    h[k] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+  }
+  double t = ((lane & 4) ? h[1] : h[0]) + __shfl_xor_sync(0xffffffffu, (lane & 4) ? h[0] : h[1], 4);
+  t += __shfl_xor_sync(0xffffffffu, t, 2);
+  t += __shfl_xor_sync(0xffffffffu, t, 1);
+  const int quantity = lane >> 2;   // bits 4, 3, 2 of the lane
+  if ((lane & 3) == 0 && quantity < 6) s_red[warp][quantity] = t;
   __syncthreads();
   if (warp == 0) {
     // lane k < 6 sums quantity k over the warps in order; lane q < 3 forms Zq of its quantity (the
     // three divisions and square roots side by side), lane 0 sums w_q Zq in the order q = 0, 1, 2
-    double t = 0.0;
+    t = 0.0;
     if (lane < 6) {
       t = s_red[0][lane];
       for (int w = 1; w < kFinWarps; ++w) t += s_red[w][lane];

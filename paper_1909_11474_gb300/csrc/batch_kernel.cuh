@@ -111,9 +111,8 @@ template <typename R>
 struct AtomAcc {
   R U, W[6];
 };
-// What the sums W are to be multiplied with to give the virial (see atom_core_f64).
-template <typename R>
-constexpr R kVirialScale = sizeof(R) == 8 ? R(-2) : R(1);
+// What the sums W = sum u (x) T are to be multiplied with to give the virial (see atom_core).
+constexpr int kVirialScale = -2;
 // FP64: the parameter set's constants in fixed point (per lane) and the tables of fx64.cuh; nothing in FP32.
 template <typename R>
 struct LaneOrder {};
@@ -169,159 +168,52 @@ __device__ __forceinline__ void stage_load(const R *stage, int row, int pl, R &x
   stage_load_row<PT, R>(stage + (size_t)row * stage_stride<PT>(), pl, x, y, z, site);
 }
 
-// The per-atom core of passes 1 and 2: from the bond geometry (unit vectors, r, 2/r, f_C, f_C', the
-// cosines of the bond pairs; R) and the parameter constants (T = R), U = sum_j f_C (f_R - b f_A), which is twice the site energy U_i of Eq. 2,
-// and P_ij = dU_i/dd_ij of every bond (the derivative of U_i itself, 1/2 included). INNER: every bond
-// is inside R1 (callers pass f_C = 1 and f_C' = 0 as constants, which the compiler folds away).
+// The per-atom core of passes 1 and 2 in FP32: from the bond geometry (unit vectors, r, f_C, f_C', the cosines of the
+// bond pairs) and the parameter constants, U = sum_j f_C (f_R - b f_A), which is twice the site energy U_i of Eq. 2,
+// and T_j = (r_j/2) dU_i/dd_ij of every bond (the derivative of U_i itself, 1/2 included):
+//   T_j = (r_j rad_j / 2 - u_j . A_j) u_j + A_j,   P_ij = (2/r_j) T_j,   -d_ij (x) P_ij = -2 u_j (x) T_j,
+// with A_j = sum_k (w_jk / 2) u_k, s_ij = sum_k w_jk cos_jk = 2 u_j . A_j since cos_jk = u_j . u_k. The virial then
+// needs neither d_ij nor P_ij. INNER: every bond is inside R1 (callers pass f_C = 1 and f_C' = 0 as constants, which
+// the compiler folds away).
 //
-// Per bond, with h_A = f_A/2 = D0 x and u2 = 2 (1 + zeta^n):
+// Per bond, with h_A = f_A/2 = D0 x, v = cos - h and u2 = 2 (1 + zeta^n):
+//   minimal form: zeta = beta sum_k f_C v^2, the factor applied once a bond; g'/2 = beta v likewise, by way of c,
 //   b = 2^(-(log2 u2 - 1)/(2n)),   f_R - b f_A = f_R - 2 b h_A,
 //   c_ij = dU_i/dzeta_ij = -1/2 f_C f_A b' = f_C (b h_A) zeta^n / (zeta u2),
 //   rad_ij = 1/2 [f_C' (f_R - b f_A) + f_C (f_R' - b f_A')],   f_R' - b f_A' = -alpha (2 f_R - b f_A),
-// the same quantities as Eq. 3-6 and their derivatives, with the constant factors folded.
-template <int M, bool INNER, typename T, typename R, bool GEN = false>
-__device__ __forceinline__ void atom_core(const R (&ux)[M], const R (&uy)[M], const R (&uz)[M],
-                                          const R (&r)[M], const R (&ir2)[M], const R (&fc)[M],
-                                          const R (&fcp)[M], const R *cs, const PConsts<T> &K, T &U,
-                                          T (&Px)[M], T (&Py)[M], T (&Pz)[M]) {
-  // ---- pass 1: pair functions (Eq. 4-5 with Eq. 11-14 at S = 2) and zeta (Eq. 7, 10)
-  constexpr int NP = M * (M - 1) / 2;
-  T fR[M], hA[M], zeta[M], tq[NP > 0 ? NP : 1];
-  T gq[GEN && NP > 0 ? NP : 1];                    // g itself (Tersoff form; the minimal form has g = t u)
-#pragma unroll
-  for (int j = 0; j < M; ++j) {
-    if constexpr (GEN) {                           // exponents of r - r0 (exact in FP32 near r0)
-      const T dr = r[j] - K.k0;
-      hA[j] = K.D0 * ex2(dr * K.k1);               // f_A / 2
-      fR[j] = K.cR * ex2(dr * K.kR1);
-    } else {                                       // x = e^{-alpha (r - r0)}; r - r0 is exact in FP32 near r0
-      const T x = ex2((r[j] - K.k0) * K.k1);
-      hA[j] = K.D0 * x;                            // f_A / 2
-      fR[j] = hA[j] * x;
-    }
-    zeta[j] = T(0.0f);
-  }
-  {
-    int q = 0;
-#pragma unroll
-    for (int j = 0; j < M; ++j) {
-#pragma unroll
-      for (int k = j + 1; k < M; ++k) {
-        const T u = cs[q] - K.h;
-        T g;
-        if constexpr (GEN) {                       // Eq. 8, in the form without cancellation
-          const T u2 = u * u;
-          const T iv = rcp(u2 + K.d2);
-          g = K.g0 + K.gcd * u2 * iv;
-          tq[q] = K.gc2 * u * iv * iv;                // g' / 2
-          gq[q] = g;
-        } else {
-          const T t = K.beta * u;                   // g = t u, g' = 2 t
-          g = t * u;
-          tq[q] = t;
-        }
-        zeta[j] += fc[k] * g;
-        zeta[k] += fc[j] * g;
-        ++q;
-      }
-    }
-  }
-  T cc[M], rad[M];
-  U = T(0.0f);
-#pragma unroll
-  for (int j = 0; j < M; ++j) {
-    const T z = zeta[j] > T(1e-30f) ? zeta[j] : T(1e-30f);   // see bond_order
-    const T zn = ex2(K.n * lg2(z));                // zeta^n
-    const T u2 = zn * R(2) + R(2);
-    const T b = ex2(K.inv2n * lg2(u2) - K.inv2n);  // (1 + zeta^n)^(-1/(2n))
-    const T bh = b * hA[j];                        // b f_A / 2
-    const T e = bh * R(-2) + fR[j];                // f_R - b f_A
-    U += fc[j] * e;                                // Eq. 3 (the 1/2 of Eq. 2 is applied by callers)
-    cc[j] = fc[j] * bh * zn * rcp(z * u2);         // dU_i / dzeta_ij
-    T mde;                                         // (f_R' - b f_A') / 2
-    if constexpr (GEN) mde = K.hl * fR[j] + K.mha * bh;   // (-lambda f_R + mu b f_A) / 2
-    else mde = K.mha * (fR[j] + e);
-    rad[j] = R(0.5) * fcp[j] * e + fc[j] * mde;
-  }
-
-  // ---- pass 2: dU_i/dd_ij
-  T Ax[M], Ay[M], Az[M], Rg[M];
-#pragma unroll
-  for (int j = 0; j < M; ++j) {
-    Ax[j] = T(0.0f); Ay[j] = T(0.0f); Az[j] = T(0.0f); Rg[j] = T(0.0f);
-  }
-  {
-    int q = 0;
-#pragma unroll
-    for (int j = 0; j < M; ++j) {
-#pragma unroll
-      for (int k = j + 1; k < M; ++k) {
-        const T w = (cc[j] * fc[k] + cc[k] * fc[j]) * tq[q];   // half of the w of the header
-        Ax[j] += w * ux[k]; Ay[j] += w * uy[k]; Az[j] += w * uz[k];
-        Ax[k] += w * ux[j]; Ay[k] += w * uy[j]; Az[k] += w * uz[j];
-        ++q;
-      }
-    }
-  }
-  // bonds inside the switching region (R1 < r < R2) carry the f_C'(r_ij) g term; the vote keeps
-  // this loop off the common path where no bond of the warp is in that region
-  bool sw = false;
-  if constexpr (!INNER) {
-#pragma unroll
-    for (int j = 0; j < M; ++j) sw |= (fcp[j] != R(0));
-    sw = __any_sync(0xffffffffu, sw);
-  }
-  if (sw) {
-    int q = 0;
-#pragma unroll
-    for (int j = 0; j < M; ++j) {
-#pragma unroll
-      for (int k = j + 1; k < M; ++k) {
-        T g;
-        if constexpr (GEN) g = gq[q];
-        else g = tq[q] * (cs[q] - K.h);
-        Rg[j] += cc[k] * g;
-        Rg[k] += cc[j] * g;
-        ++q;
-      }
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < M; ++j) {
-    // 2/r restores the factor 2 of g' = 2 t; s_ij = sum_k w_jk cos_jk = u_ij . A_ij, since
-    // cos_jk = u_ij . u_ik
-    const T sj = ux[j] * Ax[j] + uy[j] * Ay[j] + uz[j] * Az[j];
-    const T coef = rad[j] + fcp[j] * Rg[j] - sj * ir2[j];
-    Px[j] = coef * ux[j] + ir2[j] * Ax[j];
-    Py[j] = coef * uy[j] + ir2[j] * Ay[j];
-    Pz[j] = coef * uz[j] + ir2[j] * Az[j];
-  }
-}
-
-// atom_core for FP32 and the minimal form with an even neighbour bound M: the per-bond work of pass 1
-// and of the bond-order loop runs on bond pairs (2e, 2e+1) in packed FP32 pairs (two lanes of the
-// pair per instruction; the SFU operations stay scalar), the x and y components of the pass-2 sums
-// A_ij likewise; the pair loops and the final per-bond step are those of atom_core. Each packed
-// operation rounds as its scalar counterpart; only the energy sum runs in two partial sums.
+// the same quantities as Eq. 3-6 and their derivatives, with the constant factors folded. K.mha and K.hl hold half of
+// the prepared constants (tile_pass), so that `mde` is a quarter of f_R' - b f_A'.
+//
+// Even M: the per-bond work runs on bond pairs (2e, 2e+1) in packed FP32 pairs (two lanes of the pair per
+// instruction; the SFU operations stay scalar), the x and y components of A_j likewise. Each packed operation
+// rounds as its scalar counterpart; only the energy sum runs in two partial sums.
+// The loop over a warp's atoms is bound by instruction issue (the kernel issues in 52 % of the cycles, the SFU is busy
+// in a fifth of them). T_j in place of P_ij and the beta a bond instead of a pair: some 24 of an atom's 229
+// instructions less, 200 sets x 300 cells of 64 atoms 69.7 -> 68.6 us; four bonds tested ahead of the switch: 67.7 us.
 __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
 
-template <int M, bool INNER>
-__device__ __forceinline__ void atom_core_x2(const float (&ux)[M], const float (&uy)[M], const float (&uz)[M],
-                                             const float (&r)[M], const float (&ir2)[M], const float (&fc)[M],
-                                             const float (&fcp)[M], const float *cs, const PConsts<float> &K,
-                                             float &U, float (&Px)[M], float (&Py)[M], float (&Pz)[M]) {
-  static_assert(M % 2 == 0, "bond pairs");
-  constexpr int H = M / 2, NP = M * (M - 1) / 2;
-  // ---- pass 1: pair functions on bond pairs, then zeta (Eq. 7, 10) as atom_core
+template <int M, bool INNER, bool GEN>
+__device__ __forceinline__ void atom_core(const float (&ux)[M], const float (&uy)[M], const float (&uz)[M],
+                                          const float (&r)[M], const float (&fc)[M], const float (&fcp)[M],
+                                          const float *cs, const PConsts<float> &K, float &U, float (&Tx)[M],
+                                          float (&Ty)[M], float (&Tz)[M]) {
+  constexpr int H = (M + 1) / 2, NP = M * (M - 1) / 2;
+  // the second lane of the last pair of an odd M stays 0 and is not used
+  auto two = [](const auto &x, int h) { return make_float2(x[2 * h], 2 * h + 1 < M ? x[2 * h + 1 < M ? 2 * h + 1 : 0] : 0.f); };
+  auto each = [](int h, float2 t, auto &&f) { return make_float2(f(t.x), 2 * h + 1 < M ? f(t.y) : 0.f); };
+  auto exp2_2 = [&](int h, float2 t) { return each(h, t, [](float v) { return ex2(v); }); };
+  // ---- pass 1: pair functions on bond pairs, then zeta (Eq. 7, 10)
   float2 fR[H], hA[H];
 #pragma unroll
   for (int h = 0; h < H; ++h) {
-    const float2 t = __fmul2_rn(__fadd2_rn(make_float2(r[2 * h], r[2 * h + 1]), f2(-K.k0)), f2(K.k1));
-    const float2 x = make_float2(ex2(t.x), ex2(t.y));
-    hA[h] = __fmul2_rn(f2(K.D0), x);               // f_A / 2
-    fR[h] = __fmul2_rn(hA[h], x);
+    const float2 dr = __fadd2_rn(two(r, h), f2(-K.k0));              // exact near r0
+    const float2 x = exp2_2(h, __fmul2_rn(dr, f2(K.k1)));
+    hA[h] = __fmul2_rn(f2(K.D0), x);                                 // f_A / 2
+    if constexpr (GEN) fR[h] = __fmul2_rn(f2(K.cR), exp2_2(h, __fmul2_rn(dr, f2(K.kR1))));
+    else fR[h] = __fmul2_rn(hA[h], x);
   }
-  float zeta[M], tq[NP > 0 ? NP : 1];
+  float zeta[M], tq[NP > 0 ? NP : 1];                                // tq: g'/2 (minimal form: without beta)
+  float gq[GEN && NP > 0 ? NP : 1];                                  // g (Tersoff form; minimal form: tq^2)
 #pragma unroll
   for (int j = 0; j < M; ++j) zeta[j] = 0.0f;
   {
@@ -330,51 +222,68 @@ __device__ __forceinline__ void atom_core_x2(const float (&ux)[M], const float (
     for (int j = 0; j < M; ++j)
 #pragma unroll
       for (int k = j + 1; k < M; ++k) {
-        const float u = cs[q] - K.h;
-        const float t = K.beta * u;                 // g = t u, g' = 2 t
-        const float g = t * u;
-        tq[q] = t;
-        zeta[j] += fc[k] * g;
-        zeta[k] += fc[j] * g;
+        const float v = cs[q] - K.h;
+        if constexpr (GEN) {                       // Eq. 8, in the form without cancellation
+          const float v2 = v * v;
+          const float iv = rcp(v2 + K.d2);
+          const float g = K.g0 + K.gcd * v2 * iv;
+          tq[q] = K.gc2 * v * iv * iv;
+          gq[q] = g;
+          zeta[j] += fc[k] * g;
+          zeta[k] += fc[j] * g;
+        } else if constexpr (INNER) {
+          tq[q] = v;
+          zeta[j] = __fmaf_rn(v, v, zeta[j]);
+          zeta[k] = __fmaf_rn(v, v, zeta[k]);
+        } else {
+          const float v2 = v * v;
+          tq[q] = v;
+          zeta[j] = __fmaf_rn(fc[k], v2, zeta[j]);
+          zeta[k] = __fmaf_rn(fc[j], v2, zeta[k]);
+        }
         ++q;
       }
   }
   // ---- bond order and its derivative on bond pairs
-  float cc[M], rad[M];
+  float cc[M], rad[M];                             // cc: dU_i / dzeta_ij (minimal form: times beta); rad: half of it
   float2 Uh = make_float2(0.f, 0.f);
 #pragma unroll
   for (int h = 0; h < H; ++h) {
-    const float z0 = zeta[2 * h] > 1e-30f ? zeta[2 * h] : 1e-30f;
-    const float z1 = zeta[2 * h + 1] > 1e-30f ? zeta[2 * h + 1] : 1e-30f;
-    const float2 z = make_float2(z0, z1);
-    const float2 a = __fmul2_rn(f2(K.n), make_float2(lg2(z0), lg2(z1)));
-    const float2 zn = make_float2(ex2(a.x), ex2(a.y));               // zeta^n
+    float2 z = two(zeta, h);
+    if constexpr (!GEN) z = __fmul2_rn(f2(K.beta), z);
+    z = each(h, z, [](float v) { return fmaxf(v, 1e-30f); });        // see bond_order (a NaN gives 1e-30 too)
+    const float2 zn = exp2_2(h, __fmul2_rn(f2(K.n), each(h, z, [](float v) { return lg2(v); })));   // zeta^n
     const float2 u2 = __ffma2_rn(zn, f2(2.f), f2(2.f));
-    const float2 bl = __ffma2_rn(f2(K.inv2n), make_float2(lg2(u2.x), lg2(u2.y)), f2(-K.inv2n));
-    const float2 b = make_float2(ex2(bl.x), ex2(bl.y));              // (1 + zeta^n)^(-1/(2n))
-    const float2 bh = __fmul2_rn(b, hA[h]);
+    const float2 b = exp2_2(h, __ffma2_rn(f2(K.inv2n), each(h, u2, [](float v) { return lg2(v); }), f2(-K.inv2n)));
+    const float2 bh = __fmul2_rn(b, hA[h]);                          // b f_A / 2
     const float2 e = __ffma2_rn(bh, f2(-2.f), fR[h]);                // f_R - b f_A
-    const float2 zu = __fmul2_rn(z, u2);
-    float2 c = __fmul2_rn(__fmul2_rn(bh, zn), make_float2(rcp(zu.x), rcp(zu.y)));
-    const float2 mde = __fmul2_rn(f2(K.mha), __fadd2_rn(fR[h], e));
-    float2 rd;
+    float2 c = __fmul2_rn(__fmul2_rn(bh, zn), each(h, __fmul2_rn(z, u2), [](float v) { return rcp(v); }));
+    if constexpr (!GEN) c = __fmul2_rn(f2(K.beta), c);
+    float2 mde;                                                      // (f_R' - b f_A') / 4
+    if constexpr (GEN) mde = __ffma2_rn(f2(K.hl), fR[h], __fmul2_rn(f2(K.mha), bh));
+    else mde = __fmul2_rn(f2(K.mha), __fadd2_rn(fR[h], e));
+    float2 rd, eu = e;
     if constexpr (INNER) {
-      Uh = __fadd2_rn(Uh, e);
       rd = mde;
     } else {
-      const float2 fch = make_float2(fc[2 * h], fc[2 * h + 1]);
-      Uh = __ffma2_rn(fch, e, Uh);
+      const float2 fch = two(fc, h);
+      eu = __fmul2_rn(fch, e);
       c = __fmul2_rn(fch, c);
-      rd = __ffma2_rn(__fmul2_rn(f2(0.5f), make_float2(fcp[2 * h], fcp[2 * h + 1])), e, __fmul2_rn(fch, mde));
+      rd = __ffma2_rn(__fmul2_rn(f2(0.25f), two(fcp, h)), e, __fmul2_rn(fch, mde));
+    }
+    if (2 * h + 1 < M) {
+      Uh = __fadd2_rn(Uh, eu);
+      cc[2 * h + 1] = c.y;
+      rad[2 * h + 1] = rd.y;
+    } else {
+      Uh.x += eu.x;
     }
     cc[2 * h] = c.x;
-    cc[2 * h + 1] = c.y;
     rad[2 * h] = rd.x;
-    rad[2 * h + 1] = rd.y;
   }
-  U = Uh.x + Uh.y;
+  U = Uh.x + Uh.y;                                 // Eq. 3 (the 1/2 of Eq. 2 is applied by callers)
 
-  // ---- pass 2: dU_i/dd_ij (atom_core's loops, the x and y sums packed)
+  // ---- pass 2: A_j, then T_j
   float2 Axy[M];
   float Az[M], Rg[M];
 #pragma unroll
@@ -389,15 +298,16 @@ __device__ __forceinline__ void atom_core_x2(const float (&ux)[M], const float (
     for (int j = 0; j < M; ++j)
 #pragma unroll
       for (int k = j + 1; k < M; ++k) {
-        const float w = (cc[j] * fc[k] + cc[k] * fc[j]) * tq[q];
-        const float2 ww = f2(w);
-        Axy[j] = __ffma2_rn(ww, make_float2(ux[k], uy[k]), Axy[j]);
+        const float w = (cc[j] * fc[k] + cc[k] * fc[j]) * tq[q];     // half of the w of the header
+        Axy[j] = __ffma2_rn(f2(w), make_float2(ux[k], uy[k]), Axy[j]);
         Az[j] = __fmaf_rn(w, uz[k], Az[j]);
-        Axy[k] = __ffma2_rn(ww, make_float2(ux[j], uy[j]), Axy[k]);
+        Axy[k] = __ffma2_rn(f2(w), make_float2(ux[j], uy[j]), Axy[k]);
         Az[k] = __fmaf_rn(w, uz[j], Az[k]);
         ++q;
       }
   }
+  // bonds inside the switching region (R1 < r < R2) carry the f_C'(r_ij) g term; the vote keeps
+  // this loop off the common path where no bond of the warp is in that region
   bool sw = false;
   if constexpr (!INNER) {
 #pragma unroll
@@ -410,7 +320,9 @@ __device__ __forceinline__ void atom_core_x2(const float (&ux)[M], const float (
     for (int j = 0; j < M; ++j)
 #pragma unroll
       for (int k = j + 1; k < M; ++k) {
-        const float g = tq[q] * (cs[q] - K.h);
+        float g;
+        if constexpr (GEN) g = gq[q];
+        else g = tq[q] * tq[q];
         Rg[j] += cc[k] * g;
         Rg[k] += cc[j] * g;
         ++q;
@@ -419,10 +331,12 @@ __device__ __forceinline__ void atom_core_x2(const float (&ux)[M], const float (
 #pragma unroll
   for (int j = 0; j < M; ++j) {
     const float sj = ux[j] * Axy[j].x + uy[j] * Axy[j].y + uz[j] * Az[j];
-    const float coef = rad[j] + fcp[j] * Rg[j] - sj * ir2[j];
-    Px[j] = coef * ux[j] + ir2[j] * Axy[j].x;
-    Py[j] = coef * uy[j] + ir2[j] * Axy[j].y;
-    Pz[j] = coef * uz[j] + ir2[j] * Az[j];
+    float rr = rad[j];
+    if constexpr (!INNER) rr = __fmaf_rn(0.5f * fcp[j], Rg[j], rr);
+    const float coef = r[j] * rr - sj;
+    Tx[j] = __fmaf_rn(coef, ux[j], Axy[j].x);
+    Ty[j] = __fmaf_rn(coef, uy[j], Axy[j].y);
+    Tz[j] = __fmaf_rn(coef, uz[j], Az[j]);
   }
 }
 
@@ -480,10 +394,13 @@ __device__ __forceinline__ void atom_forward(const typename Vec4<R>::T *__restri
     }
   }
 
-  R U, Px[M], Py[M], Pz[M];
+  // the stage rows of this atom's bonds, and its terms of the virial added to the lane's running sums (scaled by
+  // kVirialScale at the end; a phantom bond has P = 0)
+  R U;
   if constexpr (sizeof(R) == 8) {
-    // FP64: the virial sums come with the core (W += sum u (x) T, scaled by kVirialScale at the end); short lists
-    // of which every bond of the warp is inside R1 (f_C = 1 and f_C' = 0 to the bit) fold the cutoff away
+    // FP64: the virial sums come with the core; short lists of which every bond of the warp is inside R1 (f_C = 1
+    // and f_C' = 0 to the bit) fold the cutoff away
+    R Px[M], Py[M], Pz[M];
     bool outer = !EXACT || M > 4;
     if constexpr (EXACT && M <= 4) {
 #pragma unroll
@@ -497,20 +414,25 @@ __device__ __forceinline__ void atom_forward(const typename Vec4<R>::T *__restri
     }
     if (outer)
       atom_core_f64<M, false, GEN, true>(ux, uy, uz, r, ir2, fc, fcp, cs, K, *order.lane, *order.tab, order.kc, U, acc.W, Px, Py, Pz);
-  } else if constexpr (!GEN && M % 2 == 0)
-    atom_core_x2<M, INNER>(ux, uy, uz, r, ir2, fc, fcp, cs, K, U, Px, Py, Pz);
-  else
-    atom_core<M, INNER, R, R, GEN>(ux, uy, uz, r, ir2, fc, fcp, cs, K, U, Px, Py, Pz);
-  // the stage rows of this atom's bonds, and its terms of the virial -sum_j d_ij (x) P_ij added to the
-  // lane's running sums (a phantom bond has P = 0)
 #pragma unroll
-  for (int j = 0; j < M; ++j) {
-    if (store && (EXACT || j < m)) stage_store<PT, R>(stage, lb + j, pl, Px[j], Py[j], Pz[j]);
-    if (sizeof(R) == 4 && store) {
-      const R dx = r[j] * ux[j], dy = r[j] * uy[j], dz = r[j] * uz[j];
-      acc.W[0] -= dx * Px[j]; acc.W[1] -= dy * Py[j]; acc.W[2] -= dz * Pz[j];
-      acc.W[3] -= dx * Py[j]; acc.W[4] -= dy * Pz[j]; acc.W[5] -= dz * Px[j];
+    for (int j = 0; j < M; ++j)
+      if (store && (EXACT || j < m)) stage_store<PT, R>(stage, lb + j, pl, Px[j], Py[j], Pz[j]);
+  } else {
+    float Tx[M], Ty[M], Tz[M];
+    atom_core<M, INNER, GEN>(ux, uy, uz, r, fc, fcp, cs, K, U, Tx, Ty, Tz);
+    float2 Wd = make_float2(acc.W[0], acc.W[1]);
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+      if (!store) continue;
+      if (EXACT || j < m) stage_store<PT, R>(stage, lb + j, pl, ir2[j] * Tx[j], ir2[j] * Ty[j], ir2[j] * Tz[j]);
+      Wd = __ffma2_rn(make_float2(ux[j], uy[j]), make_float2(Tx[j], Ty[j]), Wd);
+      acc.W[2] += uz[j] * Tz[j];
+      acc.W[3] += ux[j] * Ty[j];
+      acc.W[4] += uy[j] * Tz[j];
+      acc.W[5] += uz[j] * Tx[j];
     }
+    acc.W[0] = Wd.x;
+    acc.W[1] = Wd.y;
   }
   if (store) acc.U += R(0.5) * U;
 }
@@ -521,13 +443,19 @@ __device__ __forceinline__ void atom_forward_dispatch(int Mw, const typename Vec
                                                       R *stage, int lb, int lq, int m, bool store,
                                                       int pl, const PConsts<R> &K, const LaneOrder<R> &order,
                                                       AtomAcc<R> &acc) {
+  if constexpr (MMAX >= 4) {   // the diamond count ahead of the switch's jump
+    if (Mw == 4) {
+      atom_forward<4, PT, EXACT, INNER, R, GEN>(sA, sB, sC, stage, lb, lq, m, store, pl, K, order, acc);
+      return;
+    }
+  }
 #define TSF_CASE(MM)                                                                          \
   case MM:                                                                                    \
     if constexpr (MMAX >= MM)                                                                 \
       atom_forward<MM, PT, EXACT, INNER, R, GEN>(sA, sB, sC, stage, lb, lq, m, store, pl, K, order, acc); \
     break;
   switch (Mw) {
-    TSF_CASE(1) TSF_CASE(2) TSF_CASE(3) TSF_CASE(4) TSF_CASE(5) TSF_CASE(6) TSF_CASE(7) TSF_CASE(8)
+    TSF_CASE(1) TSF_CASE(2) TSF_CASE(3) TSF_CASE(5) TSF_CASE(6) TSF_CASE(7) TSF_CASE(8)
     default:
       break;
   }
@@ -776,19 +704,17 @@ template <int PTT, int MMAX, typename R, RevKind KIND, int NREV>
 __device__ __forceinline__ bool gather_pair_dispatch(int m, const R *stage, const int (&rw0)[NREV], int lb0,
                                                      const int (&rw1)[NREV], int lb1, int roff, int pl, R (&F0)[3],
                                                      R (&F1)[3]) {
-#define TSF_PCASE(MM)                                                                                    \
-  case MM:                                                                                               \
-    if constexpr (MMAX >= MM) {                                                                          \
-      gather_atom_pair<MM, PTT, R, KIND, NREV>(stage, rw0, lb0, rw1, lb1, roff, pl, F0, F1);             \
-      return true;                                                                                       \
-    }                                                                                                    \
-    return false;
-  switch (m) {
-    TSF_PCASE(3) TSF_PCASE(4)
-    default:
-      return false;
+  if constexpr (MMAX >= 4) {
+    if (m == 4) {
+      gather_atom_pair<4, PTT, R, KIND, NREV>(stage, rw0, lb0, rw1, lb1, roff, pl, F0, F1);
+      return true;
+    }
+    if (m == 3) {
+      gather_atom_pair<3, PTT, R, KIND, NREV>(stage, rw0, lb0, rw1, lb1, roff, pl, F0, F1);
+      return true;
+    }
   }
-#undef TSF_PCASE
+  return false;
 }
 
 // One parameter tile of PTT parameter sets (PTT = 32: one atom per warp; 16 or 8: 2 or 4 atoms per
@@ -833,11 +759,12 @@ __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R>
     constexpr int kStride = GEN ? 4 : 2;          // R4 records of constants per parameter set
     const R4 *kc = reinterpret_cast<const R4 *>(a.consts) + kStride * (active ? p : a.P - 1);
     const R4 k0 = kc[0], k1 = kc[1];
-    K.D0 = k0.x; K.k1 = k0.y; K.k0 = k0.z; K.mha = k0.w;
+    constexpr R kHalf = sizeof(R) == 4 ? R(0.5) : R(1);   // atom_core takes half of the derivative factors
+    K.D0 = k0.x; K.k1 = k0.y; K.k0 = k0.z; K.mha = kHalf * k0.w;
     K.beta = k1.x; K.h = k1.y; K.n = k1.z; K.inv2n = k1.w;
     if constexpr (GEN) {
       const R4 k2 = kc[2], k3 = kc[3];
-      K.cR = k2.x; K.kR1 = k2.y; K.kR0 = k2.z; K.hl = k2.w;
+      K.cR = k2.x; K.kR1 = k2.y; K.kR0 = k2.z; K.hl = kHalf * k2.w;
       K.g0 = k3.x; K.gc2 = k3.y; K.d2 = k3.z; K.gcd = k3.w;
     }
   }
@@ -993,11 +920,12 @@ __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R>
   // a fixed order. Thread (lp, k) = (tid / 8, tid % 8) of the first kNSum * PTT threads forms quantity k
   // of parameter set lp; the partials are stored [warp][lp][k ^ (lp % 8)] (the xor spreads a warp's
   // stores of one k over the banks; the reads of a row are a permutation of it).
+  static_assert(NW <= 16 && kMaxCluster <= 16, "lanes of the target norms");
   static_assert(kNSum == 8, "the reduction maps eight quantities onto eight lanes");
   R v[kNSum];
   v[0] = acc.U;
 #pragma unroll
-  for (int k = 0; k < 6; ++k) v[1 + k] = kVirialScale<R> == R(1) ? acc.W[k] : kVirialScale<R> * acc.W[k];
+  for (int k = 0; k < 6; ++k) v[1 + k] = R(kVirialScale) * acc.W[k];
   v[7] = sf;
 #pragma unroll
   for (int k = 0; k < kNSum; ++k) v[k] = sum_over_atom_slots<PTT>(v[k]);
@@ -1067,10 +995,8 @@ __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R>
       tv += __shfl_xor_sync(0xffffffffu, tv, 1);
       tv += __shfl_xor_sync(0xffffffffu, tv, 2);
       tv += __shfl_xor_sync(0xffffffffu, tv, 4);
-      const int g0 = lane & ~7;
-      const double te = __shfl_sync(0xffffffffu, term, g0);
-      const double tf = __shfl_sync(0xffffffffu, term, g0 + 7);
-      if (pp < a.P && rk < kResidualTerms) a.part[pc * kResidualTerms + rk] = rk == 0 ? te : (rk == 1 ? tv : tf);
+      static_assert(kResidualTerms == 3, "e, v, f in lanes 0, 1 and 7 of a group");
+      if (pp < a.P && (rk < 2 || rk == 7)) a.part[pc * 3 + (rk == 7 ? 2 : rk)] = rk == 1 ? tv : term;
     }
   }
   // the next tile (or item) reuses the stage, where the partial sums live. A CTA barrier suffices in
@@ -1158,16 +1084,19 @@ __global__ void __launch_bounds__(NW * kWarp, MINB) batch_kernel(const BatchPara
     // the schedule record must match the device's bond CSR: a fitness launch may be queued on the
     // previous schedule before the host has checked a rebuild's neighbour counts, and then every
     // item whose configuration changed is skipped (the host launches again on the new schedule).
-    // Every rank checks the records of all ranks of the item, so a cluster decides alike.
+    // Every warp checks the records of all ranks of the item, one a lane, so a cluster decides alike (with the
+    // records in turn, each a chain of two loads, this took 13 of 101 us for 100 cells of 64 to 512 atoms x 200 sets).
     {
       bool match = true;
-      for (unsigned r = 0; r < ncta; ++r) {
-        const CtaRec q = r == rank ? rec : a.recs[rec0 + r];
-        if (q.ns == 0) continue;
-        const int l = q.s0 + q.ns - 1, ml = a.ameta[l] & 0xffff;
-        match = match && a.boff[q.s0] == q.B0 && a.boff[l] + ml == q.B0 + q.nb && a.poff[q.s0] == q.Q0 &&
-                a.poff[l] + pair_slots(ml) == q.Q0 + q.nq;
+      if (lane < (int)ncta) {
+        const CtaRec q = a.recs[rec0 + lane];
+        if (q.ns != 0) {
+          const int l = q.s0 + q.ns - 1, ml = a.ameta[l] & 0xffff;
+          match = a.boff[q.s0] == q.B0 && a.boff[l] + ml == q.B0 + q.nb && a.poff[q.s0] == q.Q0 &&
+                  a.poff[l] + pair_slots(ml) == q.Q0 + q.nq;
+        }
       }
+      match = __all_sync(0xffffffffu, match);
       if (!match) continue;
     }
 
@@ -1287,26 +1216,12 @@ __global__ void __launch_bounds__(NW * kWarp, MINB) batch_kernel(const BatchPara
       }
     }
     const uint8_t mask = fit ? a.tmask[c] : 0;
-    if (fit && chunk == 0) {
-      // target-norm terms of Eq. 17-19 in FP64: E*^2, |W*|^2 and sum_i |F*_i|^2 (0 without the target)
-      double fsum = 0.0;
-      if (tid == 0) {
-        for (int w = 0; w < NW; ++w) fsum += s_fn[w];
-        if constexpr (CLUSTER) st_cluster(map_to_rank(smem_addr(&s_fr[rank]), 0), fsum);
-      }
-      if constexpr (CLUSTER) {
-        cluster_sync_all();
-        if (rank == 0 && tid == 0) {
-          fsum = 0.0;
-          for (unsigned r = 0; r < ncta; ++r) fsum += s_fr[r];
-        }
-      }
-      if (rank == 0 && tid == 0) {
-        double dv = 0.0;
-        for (int k = 0; k < 6; ++k) dv += a.tW[6 * (size_t)c + k] * a.tW[6 * (size_t)c + k];
-        a.dpart[3 * c] = (mask & 1) ? a.tE[c] * a.tE[c] : 0.0;
-        a.dpart[3 * c + 1] = (mask & 2) ? dv : 0.0;
-        a.dpart[3 * c + 2] = (mask & 4) ? fsum : 0.0;
+    // |F*|^2 of the slice to rank 0 of a cluster, which reads it after the tiles' cluster barriers
+    if constexpr (CLUSTER) {
+      if (fit && chunk == 0 && tid == 0) {
+        double f2 = 0.0;
+        for (int w = 0; w < NW; ++w) f2 += s_fn[w];
+        st_cluster(map_to_rank(smem_addr(&s_fr[rank]), 0), f2);
       }
     }
     const TileEnv<R> env = {stage, sA, sB, sC, satom, srev, stF, ns, s0, nat, c, cb0, B0, rec.inv_nat, s_tgt, mask,
@@ -1322,6 +1237,25 @@ __global__ void __launch_bounds__(NW * kWarp, MINB) batch_kernel(const BatchPara
       else if (kNarrow && PT > 16 && a.narrow && width <= 16)
         tile_pass<(kNarrow ? 16 : PT), PT, MMAX, CLUSTER, R, NW, GEN, FIT>(a, env, tile);
       else tile_pass<PT, PT, MMAX, CLUSTER, R, NW, GEN, FIT>(a, env, tile);
+    }
+    // target-norm terms of Eq. 17-19 in FP64: sum_i |F*_i|^2 (lanes 0-15: the warps' or ranks' sums), |W*|^2
+    // (lanes 16-23) and E*^2 (lane 24), 0 without the target. After the tiles: before them all warps waited for this
+    if (fit && chunk == 0 && rank == 0 && warp == 0) {
+      double t = 0.0;
+      if (lane < 16) {
+        if constexpr (CLUSTER) t = lane < (int)ncta ? s_fr[lane] : 0.0;
+        else t = lane < NW ? s_fn[lane] : 0.0;
+      } else if (lane < 22) {
+        t = s_tgt[lane - 15] * s_tgt[lane - 15];
+      } else if (lane == 24) {
+        t = s_tgt[0] * s_tgt[0];
+      }
+#pragma unroll
+      for (int off = 1; off < 8; off <<= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+      const double hi = __shfl_down_sync(0xffffffffu, t, 8);
+      if (lane == 0) a.dpart[3 * c + 2] = (mask & 4) ? t + hi : 0.0;
+      if (lane == 16) a.dpart[3 * c + 1] = (mask & 2) ? t : 0.0;
+      if (lane == 24) a.dpart[3 * c] = (mask & 1) ? t : 0.0;
     }
   }
 }

@@ -431,3 +431,29 @@ def test_fp64_tiles_and_parameter_ranges(P, form):
             for k in np.flatnonzero(x[:P, 3] > 0):
                 assert (got[k] - ref[k]).abs().max() <= 1e-10 * ref[k].abs().max(), (k, x[k])
     assert ctx.get_status() == 0
+
+
+@pytest.mark.parametrize("k,tol", [(-105, 1e-10), (-90, 1e-13), (100, 1e-13), (118, 1e-13)])
+def test_fp32_results_scale_with_a_power_of_two(ctx, k, tol):
+    """D0 times 2^k multiplies every FP32 quantity of the energies, forces and virials by 2^k exactly, so the results are
+    those of k = 0 times 2^k. The partial sums of a tile are added in FP32 splits for exponents from -95 to 123 and in
+    64-bit integers outside; the FP64 results then differ by their last rounding, and for k = -105 by FP32 subnormals
+    (2^-149 an operation against sums above 2^-105: 2^-44 each). Cells without bonds sum zeros in both."""
+    pos, box = [], []
+    for s in (I.workload_ga_batch(P=1, C=3)["configs"], _special_set()):
+        for c in range(s.C):
+            pos.append(s.config(c)[0])
+            box.append(s.config(c)[1])
+    cs = I.pack_configs(pos, box)
+    _build(ctx, cs)
+    params = np.tile(I.TABLE2_PARAMS, (9, 1)) * np.linspace(0.97, 1.03, 9)[:, None]
+    scaled = params.copy()
+    scaled[:, 0] *= 2.0 ** k
+    out = []
+    for x in (params, scaled):
+        E, F, W = ctx.eval(torch.tensor(x, dtype=torch.float64, device="cuda"), precision=32)
+        torch.cuda.synchronize()
+        out.append((E.cpu().numpy(), F.cpu().double().numpy(), W.cpu().numpy()))
+    assert ctx.get_status() == 0
+    for a, b, t in zip(out[0], out[1], (tol, 1e-6, tol)):
+        assert np.abs(b * 2.0 ** -k - a).max() <= t * np.abs(a).max()
