@@ -91,10 +91,9 @@ typedef struct {
  * FP64 on the first FP64 evaluation) and the evaluation schedule.
  * The build runs as one kernel queued on `stream` (one CTA per configuration), which copies pos/box
  * into the context: the caller's pos/box must stay unchanged until that kernel has run (stream order
- * suffices). The call returns once the work is queued. The neighbour counts come back to the host on
- * a side stream that waits for the kernel, so that work the caller queues next on `stream` does not
- * wait for the copy; the next call that uses the build (evaluation, fitness, gradient, export,
- * build_info) waits for the counts, checks them and builds the schedule; a rebuild of configurations
+ * suffices). The call returns once the work is queued. The kernel leaves the neighbour counts in
+ * pinned host memory; the next call that uses the build (evaluation, fitness, gradient, export,
+ * build_info) waits for the kernel, checks them and builds the schedule; a rebuild of configurations
  * of the same sizes whose neighbour counts are all unchanged reuses the previous schedule. All
  * device memory of the build (the FP64 geometry records included) is allocated by this call.
  * R1 < R2 (Eq. 9; Sec. II.B uses R1 = 2.8, R2 = 3.2). 1 <= max_nbr <= 32 bounds the entries kept

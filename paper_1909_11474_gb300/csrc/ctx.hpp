@@ -191,11 +191,9 @@ struct Ctx {
   int M = 0, max_m = 0;
   double R1 = 0, R2 = 0;
   std::vector<int> h_atom_off, h_cnt, h_m, h_boff, h_poff, h_cfg_maxm;   // host mirror of the build's layout
-  PinnedBuf hp_stage;   // pinned staging: atom table uploads, neighbour-count readback, offsets
-  cudaEvent_t stage_event = nullptr;   // recorded after the staging buffer's last upload
+  PinnedBuf hp_stage;   // pinned staging: atom table uploads, then the bond counts and error flags the build kernel writes
+  cudaEvent_t stage_event = nullptr;   // recorded on the caller's stream after the build kernel
   DevBuf atom_off, atom_cfg, pos, box, cnt, nbr, shift, boff, poff, brev;
-  cudaStream_t copy_stream = nullptr;   // the build's count readback runs here, beside later calls
-  cudaEvent_t build_done = nullptr;     // recorded after the build kernel on the caller's stream
   DevBuf counters;   // per-launch work counters of the persistent batched kernels
   DevBuf gA32, gB32, gcos32, gA64, gB64, gcos64;
   DevBuf ameta;   // [Ntot] int: bonds kept (min(cnt, M)) | (some bond beyond R1, f_C != 1) << 16
@@ -241,7 +239,8 @@ struct BuildLaunch {
   float *gcos;
   int *ameta;
   int4 *arev;
-  unsigned *status, *build_status;   // the context's status word and the build's own
+  unsigned *status;                // the context's status word
+  int *h_cnt, *h_flag;             // pinned host memory the kernel writes (BuildParams)
   int nat_max;    // largest configuration (atoms)
 };
 cudaError_t launch_build_batch(const BuildLaunch &L, cudaStream_t s);

@@ -198,7 +198,8 @@ struct BuildParams {
   float *gcos;
   int *ameta;                      // [Ntot]: bonds kept (min(cnt, M)) | (some bond beyond R1) << 16
   int4 *arev;                      // [Ntot]: configuration-local reverse bonds of the first 8 bonds, 16 bits each
-  unsigned *status, *build_status; // the context's status word and the build's own (read by the host)
+  unsigned *status;                // the context's status word
+  int *h_cnt, *h_flag;             // pinned host memory: bonds kept of every atom; [0] set on non-finite input, [1] on an overflow
   int nat_max;                     // largest configuration of the launch (shared-memory layout)
   int lists_in_smem;               // the lists and unit vectors fit in shared memory
   int pairmask;                    // the pair-membership bit matrix fits in shared memory (at pm_off)
@@ -208,7 +209,7 @@ struct BuildParams {
 
 __device__ __forceinline__ void build_flag(const BuildParams &a, unsigned bit) {
   set_status(a.status, bit);
-  set_status(a.build_status, bit);
+  a.h_flag[bit == TERSOFF_STATUS_NONFINITE ? 0 : 1] = 1;
 }
 
 // Dynamic shared memory of the build kernel for configurations of up to nat atoms.
@@ -624,6 +625,7 @@ __global__ void __launch_bounds__(kBuildThreads, 2) build_batch_kernel(const Bui
   for (int t = tid; t < nat; t += kBuildThreads) {
     a.boff[a0 + t] = (int)(base_b + s_boff[t]);
     a.poff[a0 + t] = (int)(base_q + s_poff[t]);
+    a.h_cnt[a0 + t] = s_m[t];   // to the host as they stand: a copy queued after the kernel took two more launches
   }
   // one thread per bond: owner atom, reverse entry (j; i, -n), record
   for (int bl = tid; bl < nb; bl += kBuildThreads) {
@@ -750,7 +752,8 @@ cudaError_t launch_build_batch(const BuildLaunch &L, cudaStream_t s) {
   a.ameta = L.ameta;
   a.arev = L.arev;
   a.status = L.status;
-  a.build_status = L.build_status;
+  a.h_cnt = L.h_cnt;
+  a.h_flag = L.h_flag;
   a.nat_max = std::max(1, L.nat_max);
   const size_t base = (build_smem_base(a.nat_max) + 15) / 16 * 16;
   const size_t with_lists = base + build_smem_lists(a.nat_max, L.M);

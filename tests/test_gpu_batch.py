@@ -457,3 +457,41 @@ def test_fp32_results_scale_with_a_power_of_two(ctx, k, tol):
     assert ctx.get_status() == 0
     for a, b, t in zip(out[0], out[1], (tol, 1e-6, tol)):
         assert np.abs(b * 2.0 ** -k - a).max() <= t * np.abs(a).max()
+
+
+@pytest.mark.parametrize("change", ["none", "counts", "overflow", "nonfinite"])
+@pytest.mark.parametrize("C", [1, 6])
+def test_eval_queued_before_rebuild_check(change, C):
+    """An FP32 evaluation right after a rebuild of the same layout is queued before the host has read the counts and
+    error flags that the build kernel leaves in pinned memory. Its results equal those of a fresh context built once on
+    the new positions, and the build's errors come back from it."""
+    from paper_1909_11474_gb300 import binding
+    w = I.workload_ga_batch(P=9, C=C)
+    cs = w["configs"]
+    params = torch.tensor(w["params"], device="cuda")
+    c = binding.Context(0)
+    _build(c, cs)
+    c.eval(params)
+    pos2 = cs.pos.copy() + np.random.default_rng(4).normal(0, 0.01, cs.pos.shape)
+    a0 = cs.atom_off[C - 1]
+    if change == "counts":
+        pos2[a0] += 0.7 * np.array([1.0, 1.0, 0.0]) / np.sqrt(2.0)
+    if change == "overflow":                  # 33 atoms within a sphere of radius 0.8
+        d = np.random.default_rng(1).normal(size=(33, 3))
+        pos2[a0:a0 + 33] = pos2[a0] + 0.8 * d / np.linalg.norm(d, axis=1)[:, None]
+    if change == "nonfinite":
+        pos2[a0, 1] = np.nan
+    p2, b2 = torch.tensor(pos2, device="cuda"), torch.tensor(cs.box, device="cuda")
+    c.build_neighbors(cs.atom_off, p2, b2, 2.8, 3.2, 16)
+    if change in ("overflow", "nonfinite"):
+        with pytest.raises(binding.TersoffError) as ei:
+            c.eval(params)
+        assert ei.value.code == (binding.E_NBR_OVERFLOW if change == "overflow" else binding.E_NONFINITE)
+        return
+    got = c.eval(params)
+    torch.cuda.synchronize()
+    assert c.get_status() == 0
+    fresh = binding.Context(0)
+    fresh.build_neighbors(cs.atom_off, p2, b2, 2.8, 3.2, 16)
+    for a, b in zip(got, fresh.eval(params)):
+        assert torch.equal(a, b)
