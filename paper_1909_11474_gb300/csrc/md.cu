@@ -1068,26 +1068,6 @@ __device__ __forceinline__ void md_force_atom64(int N, int M, int i, int m, cons
   }
 }
 
-// Warp sums of eight values: each step sends half of the values to the other half of the lanes, so that 9 additions do
-// what a butterfly of every value takes 40 for (the FP64 unit issues an addition in 64 cycles a scheduler). Lane l with
-// l % 4 = 0 ends with the sum of value 4 (l / 16) + 2 (l / 8 % 2) + (l / 4 % 2).
-__device__ __forceinline__ double md_warp_sums(double (&v)[8]) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int h = 4; h >= 1; h >>= 1) {
-    const int off = 4 * h;
-    const bool up = (lane & off) != 0;
-#pragma unroll
-    for (int k = 0; k < h; ++k) {
-      const double send = up ? v[k] : v[k + h], keep = up ? v[k + h] : v[k];
-      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-    }
-  }
-  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
-  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
-  return v[0];
-}
-
 // Four lanes an atom, a lane a bond. A scheduler's FP64 unit takes 64 cycles a warp instruction, so what counts for a
 // small system is how many schedulers have work and how few FP64 instructions stand in one warp's line: 4,096 atoms reach
 // 512 schedulers with ~65 each instead of 128 with ~300 (51.2 us with the library's functions and a thread an atom, 32 us
@@ -1132,7 +1112,7 @@ __global__ void __launch_bounds__(kMdThreads, 4) md_force64_kernel(
   }
   // per-warp sums, per-block FP64 partial sums of U_i = U/2 and W = -2 Wv, stored [7][blocks]
   double v[8] = {U, Wv[0], Wv[1], Wv[2], Wv[3], Wv[4], Wv[5], 0.0};
-  const double t = md_warp_sums(v);
+  const double t = warp_sums8(v);
   if ((tid & 3) == 0) red[tid >> 5][(tid >> 2) & 7] = t;
   __syncthreads();
   const int nblk = gridDim.x, b = blockIdx.x;
