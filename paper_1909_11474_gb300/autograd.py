@@ -11,7 +11,7 @@ class TersoffLoss(torch.autograd.Function):
     """L[p] = loss of parameter set p over the context's configurations and targets.
 
     forward(params [P][6] float64 CUDA, ctx, targets, w, loss) -> L [P]; backward gives
-    dL/dparams = grad_L[p] * dL[p]/dx from the library's adjoint kernel.
+    dL/dparams = grad_L[p] * dL[p]/dx from tersoff_param_grad.
     """
 
     @staticmethod

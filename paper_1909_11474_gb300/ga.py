@@ -5,7 +5,7 @@ Each generation evaluates the fitness Z of the whole population with `Context.fi
 next population with one `tersoff_ga_step` kernel (rank, elite, parents, uniform crossover,
 mutation); the uniform random numbers come from a seeded torch generator on the device. Nothing is
 copied to the host inside the loop. A run can be saved and resumed bit for bit (`save`, `load`).
-`polish` then refines the best parameter set with the adjoint gradient of the smooth loss
+`polish` then refines the best parameter set with the gradient of the smooth loss
 (`TersoffLoss`), the use the gradient kernel serves beside the GA.
 """
 from __future__ import annotations
@@ -113,7 +113,7 @@ class GeneticFit:
 
 def _newton_polish(ctx, g0, lo, hi, targets, w, loss, iters: int, h: float = 1e-4):
     """Damped Newton (Levenberg-Marquardt damping) in gene space. Each iteration evaluates the loss
-    and its adjoint gradient at the point and at +-h along every gene in one batched call (13
+    and its gradient at the point and at +-h along every gene in one batched call (13
     parameter sets), takes the Hessian by central differences of the gradients, and solves the 6x6
     system (H + lam diag(H)) d = -grad on the host; a step that lowers the loss is taken and lam
     shrinks, else lam grows. Stops when two accepted steps in a row gain less than 1e-10 relative."""
@@ -236,9 +236,9 @@ def _fd_newton_polish(ctx, g0, lo, hi, targets, w, iters: int, h: float = 1e-4):
 def polish(ctx: binding.Context, params, targets: dict, lo, hi, steps: int = 30, lr: float = 2e-3,
            w=(1.0, 1.0, 1.0), loss: int = binding.LOSS_SQ, method: str = "auto"):
     """Refine one parameter set on the smooth loss L = sum_q w_q S_q / D_q in gene space, with
-    gradients from the adjoint kernel. The loss is a least-squares sum whose six directions are
+    gradients from tersoff_param_grad. The loss is a least-squares sum whose six directions are
     badly scaled (beta and n trade off along a long valley), so the default is a damped Newton method
-    on a finite-difference Hessian of the adjoint gradient (`steps` iterations, one batched call of
+    on a finite-difference Hessian of the gradient (`steps` iterations, one batched call of
     13 parameter sets each); `method="lbfgs"` (strong-Wolfe line search) and `method="adam"` (rate
     `lr`) are first-order alternatives. With `method="fd-newton"` the damped Newton step takes its
     gradient and Hessian by central differences of the FP64 fitness instead (no gradient kernel).
