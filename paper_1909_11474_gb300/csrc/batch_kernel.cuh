@@ -1097,7 +1097,11 @@ __global__ void __launch_bounds__(NW * kWarp, MINB) batch_kernel(const BatchPara
         }
       }
       match = __all_sync(0xffffffffu, match);
-      if (!match) continue;
+      if (!match) {
+        // every warp of every rank comes here; none may still have to read s_item when the next item is claimed
+        if constexpr (CLUSTER) cluster_sync_all(); else __syncthreads();
+        continue;
+      }
     }
 
     // atom slice of this CTA

@@ -495,3 +495,35 @@ def test_eval_queued_before_rebuild_check(change, C):
     fresh.build_neighbors(cs.atom_off, p2, b2, 2.8, 3.2, 16)
     for a, b in zip(got, fresh.eval(params)):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("call", ["eval", "fitness"])
+@pytest.mark.parametrize("C,reps", [(700, (1, 1, 1)), (120, (4, 4, 3))])
+def test_stale_items_are_skipped_in_runs(call, C, reps):
+    """A rebuild that changes the counts of nearly every configuration: the call queued ahead of the check skips one item
+    after another (on single CTAs and on clusters, several items each), and its results are those of a fresh context."""
+    from paper_1909_11474_gb300 import binding
+    rng = np.random.default_rng(8)
+    cs = I.make_cells(rng, C, lambda: reps, lambda: I.random_strain(rng, 0.01), lambda: 0.05, lambda: 0)
+    pos2 = cs.pos.copy()
+    for k in range(C):
+        if k % 16:                            # one atom moved by 0.7 A along <110> gains second-shell bonds
+            pos2[cs.atom_off[k]] += 0.7 * np.array([1.0, 1.0, 0.0]) / np.sqrt(2.0)
+    t = {"E": np.full(cs.C, -4.6), "W": np.zeros((cs.C, 6)), "F": np.zeros((cs.Ntot, 3)),
+         "mask": np.full(cs.C, 7, np.uint8)}
+    params, tg = torch.tensor(I.population(rng, 37)[0], device="cuda"), targets_to_device(t)
+    run = (lambda c: c.eval(params)) if call == "eval" else (lambda c: c.fitness(params, tg))
+    pos, box = to_device(cs)
+    new = torch.tensor(pos2, device="cuda")
+    c = binding.Context(0)
+    for x in (pos, new, pos):
+        c.build_neighbors(cs.atom_off, x, box, 2.8, 3.2, 16)
+        got = run(c)
+        assert c.get_status() == 0
+        fresh = binding.Context(0)
+        fresh.build_neighbors(cs.atom_off, x, box, 2.8, 3.2, 16)
+        for u, v in zip(got, run(fresh)):
+            assert torch.equal(u, v)
+        counts = c.export_neighbors()[0]
+        assert x is not new or (np.add.reduceat(counts, cs.atom_off[:-1]) != before).sum() > 0.5 * C
+        before = np.add.reduceat(counts, cs.atom_off[:-1])
