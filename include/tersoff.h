@@ -94,7 +94,9 @@ typedef struct {
  * suffices). The call returns once the work is queued. The kernel leaves the neighbour counts in
  * pinned host memory; the next call that uses the build (evaluation, fitness, gradient, export,
  * build_info) waits for the kernel, checks them and builds the schedule; a rebuild of configurations
- * of the same sizes whose neighbour counts are all unchanged reuses the previous schedule. All
+ * of the same sizes whose neighbour counts are all unchanged reuses the previous schedule. That call
+ * may be on another stream: its work runs after the build kernel (FP32 evaluations and fitness calls
+ * after a rebuild of the same sizes are queued behind it before the host waits, others after). All
  * device memory of the build (the FP64 geometry records included) is allocated by this call.
  * R1 < R2 (Eq. 9; Sec. II.B uses R1 = 2.8, R2 = 3.2). 1 <= max_nbr <= 32 bounds the entries kept
  * per atom. Argument errors are returned by this call. Errors found by the build kernel are

@@ -641,10 +641,22 @@ static int queue_eval(tersoff_ctx *ctx, const double *params, int32_t P, int32_t
 }
 
 // Whether an FP32 call may be queued on the previous schedule before the host has checked a rebuild's counts: see
-// tersoff_fitness.
-static bool may_speculate(const Ctx &c, int precision) {
-  return c.pending && c.pending_same_layout && precision == 32 && c.plan32.precision == 32 && !c.plan32.buckets.empty() &&
-         c.max_m <= 8;
+// tersoff_fitness. Then `stream`, which need not be the build's, goes on after the build kernel: until the host waits for
+// it, nothing else orders the two. (A stream that is being captured cannot take an order on work outside its graph: there
+// the host waits first.)
+static int may_speculate(tersoff_ctx *ctx, int precision, cudaStream_t stream, bool *yes) {
+  const Ctx &c = ctx->c;
+  *yes = false;
+  if (!(c.pending && c.pending_same_layout && precision == 32 && c.plan32.precision == 32 && !c.plan32.buckets.empty() &&
+        c.max_m <= 8))
+    return TERSOFF_OK;
+  TSF_CUDA(cudaSetDevice(c.device));
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  TSF_CUDA(cudaStreamIsCapturing(stream, &cap));
+  if (cap != cudaStreamCaptureStatusNone) return TERSOFF_OK;
+  TSF_CUDA(cudaStreamWaitEvent(stream, c.stage_event, 0));
+  *yes = true;
+  return TERSOFF_OK;
 }
 
 int tersoff_eval(tersoff_ctx *ctx, const double *params, int32_t P, int32_t precision, double *E,
@@ -654,7 +666,10 @@ int tersoff_eval(tersoff_ctx *ctx, const double *params, int32_t P, int32_t prec
   const bool args = params && P >= 1 && (precision == 32 || precision == 64);
   // queued ahead of the check of a rebuild as in tersoff_fitness: one 64-atom cell rebuilt and evaluated for 8 sets
   // took 43 us of library calls when the counts were waited for first, 27 us now
-  if (args && may_speculate(c, precision)) {
+  bool ahead = false;
+  if (args)
+    if (int rc = may_speculate(ctx, precision, S(stream), &ahead)) return rc;
+  if (ahead) {
     const uint64_t gen = c.plan32.gen;
     if (int rc = queue_eval(ctx, params, P, precision, E, F, W, stream)) return rc;
     if (int rc = tsf::finish_build(ctx)) return rc;
@@ -683,7 +698,9 @@ int tersoff_fitness(tersoff_ctx *ctx, const double *params, int32_t P, const ter
   // no longer matches the device's bond CSR; if the counts did change, the host (which then drains
   // the device before rebuilding the schedule) clears the status bits of that launch and queues the
   // call again on the new schedule.
-  if (may_speculate(c, precision)) {
+  bool ahead = false;
+  if (int rc = may_speculate(ctx, precision, S(stream), &ahead)) return rc;
+  if (ahead) {
     const uint64_t gen = c.plan32.gen;
     if (int rc = queue_fitness(ctx, params, P, tg, w, precision, Z, Zq, Sq, stream)) return rc;
     if (int rc = tsf::finish_build(ctx)) return rc;

@@ -527,3 +527,63 @@ def test_stale_items_are_skipped_in_runs(call, C, reps):
         counts = c.export_neighbors()[0]
         assert x is not new or (np.add.reduceat(counts, cs.atom_off[:-1]) != before).sum() > 0.5 * C
         before = np.add.reduceat(counts, cs.atom_off[:-1])
+
+
+@pytest.mark.parametrize("call", ["eval", "fitness"])
+@pytest.mark.parametrize("change_counts", [False, True])
+def test_rebuild_on_one_stream_and_call_on_another(call, change_counts):
+    """A rebuild queued on one stream behind 20 ms of other work, and the FP32 call that uses it on another stream: the
+    call's results are those of a fresh context built on the new positions, not of the old or a half-written geometry."""
+    from paper_1909_11474_gb300 import binding
+    w = I.workload_ga_batch(P=37, C=40)
+    cs = w["configs"]
+    t = {"E": np.full(cs.C, -4.6), "W": np.zeros((cs.C, 6)), "F": np.zeros((cs.Ntot, 3)),
+         "mask": np.full(cs.C, 7, np.uint8)}
+    params, tg = torch.tensor(w["params"], device="cuda"), targets_to_device(t)
+    c = binding.Context(0)
+    run = (lambda c: c.eval(params)) if call == "eval" else (lambda c: c.fitness(params, tg))
+    pos, box = to_device(cs)
+    pos2 = cs.pos + np.random.default_rng(4).normal(0, 0.01, cs.pos.shape)
+    if change_counts:
+        pos2[cs.atom_off[3]] += 0.7 * np.array([1.0, 1.0, 0.0]) / np.sqrt(2.0)
+    new = torch.tensor(pos2, device="cuda")
+    fresh = binding.Context(0)
+    fresh.build_neighbors(cs.atom_off, new, box, 2.8, 3.2, 16)
+    want = run(fresh)
+    c.build_neighbors(cs.atom_off, pos, box, 2.8, 3.2, 16)
+    run(c)
+    torch.cuda.synchronize()
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    with torch.cuda.stream(a):
+        torch.cuda._sleep(int(0.02 * 2e9))
+        c.build_neighbors(cs.atom_off, new, box, 2.8, 3.2, 16)
+    with torch.cuda.stream(b):
+        got = run(c)
+    torch.cuda.synchronize()
+    assert c.get_status() == 0
+    for x, y in zip(got, want):
+        assert torch.equal(x, y)
+
+
+def test_evaluation_captured_right_after_a_rebuild():
+    """A stream under capture cannot be ordered after the build on a stream outside: the host waits first, and the graph
+    holds the evaluation of the new positions."""
+    from paper_1909_11474_gb300 import binding
+    cs = I.workload_ga_batch(P=1, C=3)["configs"]
+    params = torch.tensor(I.population(np.random.default_rng(2), 9)[0], device="cuda")
+    c = binding.Context(0)
+    pos, box = to_device(cs)
+    c.build_neighbors(cs.atom_off, pos, box, 2.8, 3.2, 16)
+    c.eval(params)
+    new = pos + 0.01 * torch.randn(pos.shape, dtype=torch.float64, device="cuda",
+                                   generator=torch.Generator(device="cuda").manual_seed(3))
+    c.build_neighbors(cs.atom_off, new, box, 2.8, 3.2, 16)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, capture_error_mode="relaxed"):
+        got = c.eval(params)
+    g.replay()
+    torch.cuda.synchronize()
+    fresh = binding.Context(0)
+    fresh.build_neighbors(cs.atom_off, new, box, 2.8, 3.2, 16)
+    for x, y in zip(got, fresh.eval(params)):
+        assert torch.equal(x, y)
