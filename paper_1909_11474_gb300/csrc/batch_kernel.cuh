@@ -820,10 +820,11 @@ __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R>
   // ---- pass 3: F_i = sum_j (P_ij - P_ji)
   R sf = R(0);   // sum |F - F*|^2 over the warp's atoms, or sum |F|^2 without a force target
   // F of atom li in the variants with several atoms in a warp: the own and the reverse rows summed in order,
-  // as in gather_sum. Tiles of the kernel's own width find the reverse rows in srev, narrow last tiles (whose
+  // as in gather_sum; nothing for an atom with more than MMAX bonds, which pass 1 flagged (a fitness queued ahead of a
+  // rebuild's check may meet one where the totals agree: srev holds eight entries an atom). Tiles of the kernel's own width find the reverse rows in srev, narrow last tiles (whose
   // srev holds offsets in the full-width stage) in the bond record
   auto gather_loop = [&](int li, const int4 &at, R (&F)[3]) {
-    const int m = at.z, lb = at.x;
+    const int m = at.z <= MMAX ? at.z : 0, lb = at.x;
     R o[3] = {R(0), R(0), R(0)}, r[3] = {R(0), R(0), R(0)};
     for (int e = 0; e < m; ++e) {
       R x, y, z;

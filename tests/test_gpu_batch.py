@@ -587,3 +587,40 @@ def test_evaluation_captured_right_after_a_rebuild():
     fresh.build_neighbors(cs.atom_off, new, box, 2.8, 3.2, 16)
     for x, y in zip(got, fresh.eval(params)):
         assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("tile,P", [(16, 16), (16, 21), (16, 5), (32, 5), (32, 40)])
+def test_rebuild_with_a_long_list_and_equal_totals(tile, P):
+    """Three triangles and a lone atom become a star of nine bonds: bonds and pair slots of the cell stay 18 and 36, so
+    that its schedule record still matches and the fitness queued ahead of the check runs on lists longer than its
+    kernel's. It reads nothing out of range, and the call returns TERSOFF_E_UNSUPPORTED."""
+    from paper_1909_11474_gb300 import binding
+    g = (1 + 5 ** 0.5) / 2
+    ico = np.array([[0, s, t * g] for s in (1, -1) for t in (1, -1)])
+    ico = np.concatenate([ico, ico[:, [2, 0, 1]], ico[:, [1, 2, 0]]]) / np.sqrt(1 + g * g)
+    star = 20.0 + np.concatenate([3.1 * ico[:9], np.zeros((1, 3))])        # leaves 3.26 apart; the centre last
+    tri = 2.4 * np.array([[0, 0, 0], [1, 0, 0], [0.5, 0.75 ** 0.5, 0]])
+    rings = np.concatenate([tri, tri + 10.0, tri + 20.0, [[30.0, 5.0, 5.0]]])
+    box = np.eye(3) * 40.0
+    old, new = I.pack_configs([rings] * 3, [box] * 3), I.pack_configs([rings, star, rings], [box] * 3)
+    slots = lambda m: ((m * (m - 1) // 2 + 3) // 4 * 4).sum()              # noqa: E731
+    for cs, top in ((old, 2), (new, 9)):
+        m = np.diff(oracle.neighbor_list(*cs.config(1), 3.2)["off"])
+        assert (m.max(), m.sum(), slots(m)) == (top, 18, 36)
+    t = targets_to_device({"E": np.full(3, -1.0), "W": np.zeros((3, 6)), "F": np.zeros((30, 3)),
+                           "mask": np.full(3, 7, np.uint8)})
+    params = torch.tensor(I.population(np.random.default_rng(1), P)[0], device="cuda")
+    c = binding.Context(0)
+    _build(c, old)
+    c.set_schedule(P, tile=tile)
+    want = [x.cpu() for x in c.fitness(params, t)]
+    _build(c, new)
+    with pytest.raises(binding.TersoffError) as ei:
+        c.fitness(params, t)
+    assert ei.value.code == binding.E_UNSUPPORTED
+    torch.cuda.synchronize()
+    c.get_status()
+    _build(c, old)
+    for x, y in zip(c.fitness(params, t), want):
+        assert np.allclose(x.cpu(), y, rtol=1e-6)
+    assert c.get_status() == 0
