@@ -158,6 +158,8 @@ __host__ __device__ __forceinline__ int64_t fx_mul(int64_t a, int64_t b) {
   return (int64_t)(((uint64_t)TSF_SMULHI64(a, b) << (64 - S)) | (((uint64_t)a * (uint64_t)b) >> S));
 }
 
+__host__ __device__ __forceinline__ int64_t fx_add(int64_t a, int64_t b) { return (int64_t)((uint64_t)a + (uint64_t)b); }
+
 // The pair functions and the bond order of one parameter set in fixed point:
 //   f_R = 2^(lR + kR (r - r0)),   f_A / 2 = 2^(lA + kA (r - r0)),   zeta = 2^lB S,   b = (1 + zeta^n)^(-1/(2n)).
 // The minimal form has lR = lA = log2 D0, kR = 2 kA and lB = log2 beta (S the angular sum without beta). ok: every
@@ -191,16 +193,19 @@ __host__ __device__ __forceinline__ bool fx_bond(double r, double S, const FxLan
   if (!o.ok || !fx_from_double<58, 4>(r, R) || (us >> 52) > 1023u + 200u) return false;
   const int64_t lmin = -1795276095634356808ll;     // log2(1e-30) with 54 fraction bits
   int64_t L = lmin;
-  if (fx_log2_double(S, t, LS)) L = LS + o.lB > lmin ? LS + o.lB : lmin;   // S = 0, or below 2^-200: clamped
-  const int64_t dr = R - o.r0;                     // |dr| < 16
-  const int64_t YA = o.lA + fx_mul<58, 58>(dr, o.kA), YR = o.lR + fx_mul<58, 58>(dr, o.kR);
+  if (fx_log2_double(S, t, LS)) L = LS + o.lB > lmin ? LS + o.lB : lmin;
+  else if (us != 0) return false;                  // below 2^-200; S = 0 is clamped
+  if (L >= 125ll << 54) return false;              // so that n L stays below 512, which is all that fits
+  const int64_t dr = R - o.r0;                     // |dr| < 32
+  // sums of two exponents may wrap (at 512), from at most 200 + 512, to something beyond lim
+  const int64_t YA = fx_add(o.lA, fx_mul<58, 58>(dr, o.kA)), YR = fx_add(o.lR, fx_mul<58, 58>(dr, o.kR));
   const int64_t Y = fx_mul<54, 60>(L, o.n);        // n L
   const int64_t lim = 250ll << 54;
   if (Y >= lim || Y <= -lim || YA >= lim || YA <= -lim || YR >= lim || YR <= -lim) return false;
   const FxNum w = fx_one_plus(fx_exp2(Y, t));
   const int64_t L2 = fx_log2(w, t);                // 0 <= L2 < 251
-  const int64_t H = YA - fx_mul<54, 56>(L2, o.inv2n);              // log2 of b f_A / 2 (0 <= L2/(2n) < 135)
-  const int64_t C = H + (Y - L - L2 - (1ll << 54) + o.lB);
+  const int64_t H = YA - fx_mul<54, 56>(L2, o.inv2n);              // log2 of b f_A / 2 (0 <= L2/(2n) < 95)
+  const int64_t C = fx_add(H, Y - L - L2 - (1ll << 54) + o.lB);    // between -640 and 550 where H is above -lim
   if (H <= -lim || C >= lim || C <= -lim) return false;
   fR = fx_to_double(fx_exp2(YR, t));
   bh = fx_to_double(fx_exp2(H, t));

@@ -86,3 +86,49 @@ def test_fixed_point_bond_functions(tmp_path):
     assert max(worst[3:]) <= 1.5e-15, worst
     assert refused == 0 and bad == 0
     assert refused_wide < 0.05 * 200000
+
+
+RANGE_SRC = SRC[:SRC.index("int main()")] + r"""
+int main() {
+  const FxTables &t = kFxTables;
+  std::mt19937_64 g(11);
+  std::uniform_real_distribution<double> U(-1, 1);
+  auto pow2 = [&](double top) { return std::exp2(top * U(g)); };
+  long taken = 0, wrong = 0;
+  for (int i = 0; i < 2000000; ++i) {
+    const double D0 = pow2(i & 1 ? 201 : 20), be = pow2(i & 2 ? 201 : 20), n = i & 4 ? 2 + 2 * U(g) : 0.3 + 0.29 * U(g);
+    const double r0 = 16 * U(g), r = 8 + 8 * U(g), k = i & 8 ? 16 * U(g) : 2 * U(g), in = -0.5 / n;
+    double S = i & 16 ? pow2(201) : pow2(20);
+    if (i % 31 == 0) S = std::ldexp(1 + 0.5 * U(g), -150 - i % 925);         // down to subnormals
+    if (i % 37 == 0) S = 0;
+    double fR, bh, cc;
+    if (!fx_bond(r, S, fx_lane(r0, k, 2 * k, D0, D0, be, n, in, t), t, fR, bh, cc)) continue;
+    ++taken;
+    const Q x = std::exp2((Q)k * ((Q)r - (Q)r0)), hA = D0 * x;
+    Q z = (Q)be * (Q)S;
+    if (z < (Q)1e-30) z = 1e-30;
+    const Q zn = std::exp2((Q)n * std::log2(z)), b = std::exp2((Q)in * std::log2(1 + zn));
+    const Q ref[3] = {hA * x, b * hA, (Q)be * b * hA * (zn / (1 + zn)) / (2 * z)};
+    const double got[3] = {fR, bh, cc};
+    for (int q = 0; q < 3; ++q) wrong += !(std::fabs((got[q] - ref[q]) / ref[q]) <= (Q)1e-14);
+  }
+  double a, b, c;   // zeta = 2^262, n = 3.9: zeta^n is far outside, b f_A / 2 is 1.0e-39
+  wrong += fx_bond(2.35, std::ldexp(1, 63), fx_lane(2.35, -2, -4, 3.2, 3.2, std::ldexp(1, 199), 3.9, -0.5 / 3.9, t), t, a, b, c);
+  std::printf("%ld %ld\n", taken, wrong);
+}
+"""
+
+
+def test_fixed_point_bond_functions_at_the_ends_of_their_ranges(tmp_path):
+    """Whatever is not refused is right, at the ends of every range that fx_lane and fx_bond accept. The exponents err by at
+    most 2^-46.6 (1/(2n) <= 32 times the errors of n L and of log2(1 + zeta^n), and log2(1 + zeta^n) <= 250 times the
+    2^-56 to which 1/(2n) is held), the values by ln2 times that, 6.5e-15, and cc by another 2^-49."""
+    cxx = shutil.which("g++")
+    if cxx is None:
+        pytest.skip("no g++")
+    src = tmp_path / "fxr.cpp"
+    src.write_text(RANGE_SRC)
+    exe = tmp_path / "fxr"
+    subprocess.run([cxx, "-O2", "-std=c++17", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    taken, wrong = (int(x) for x in subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split())
+    assert taken > 200000 and wrong == 0, (taken, wrong)
