@@ -31,6 +31,7 @@ def nvcc() -> str:
 
 def _deps() -> list[str]:
     return (glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.hpp"))
+            + glob.glob(os.path.join(CSRC, "*.inc"))
             + [os.path.join(ROOT, "include", "tersoff.h")])
 
 

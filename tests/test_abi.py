@@ -45,3 +45,13 @@ def test_binding_loads_library_and_sets_signatures(lib):
     # null context is rejected on the host before any CUDA call
     assert L.tersoff_eval(None, None, 1, 32, None, None, None, None) == binding.E_ARG
     assert L.tersoff_last_error(None) == b""
+
+
+def test_build_watches_every_included_file():
+    """Each file that a source of the library includes is one whose change makes the objects stale."""
+    from paper_1909_11474_gb300 import build
+    deps = {os.path.realpath(d) for d in build._deps()}
+    for name in os.listdir(build.CSRC):
+        path = os.path.join(build.CSRC, name)
+        for inc in re.findall(r'^\s*#include "([^"]+)"', open(path).read(), re.M):
+            assert os.path.realpath(os.path.join(build.CSRC, inc)) in deps, f"{name} includes {inc}"
