@@ -1377,7 +1377,7 @@ __global__ void md_accel_kernel(int N, const double *__restrict__ mass, double *
 }
 
 // One step's per-atom work between two searches, in one kernel: F_i from the P_ij (md_gather_kernel), the second half
-// kick v += a F h of the step just evaluated (h = 0 before the first), the kinetic energy sum_i m v^2 / 2 into *Ekin
+// kick v += a F h of the step just evaluated (none before the first), the kinetic energy sum_i m v^2 / 2 into *Ekin
 // in a fixed order, and, but after the last step, the first half kick v += a F dt/2 and the drift x += v dt of the
 // next one with the binning of the new position. Every part is local to the atom, so a step is three launches
 // (search, force, this) instead of eight with two memsets.
@@ -1400,7 +1400,8 @@ __global__ void __launch_bounds__(kMdThreads) md_advance_kernel(
     double v[3], v2 = 0.0;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      v[k] = vel[3 * i + k] + h * (double)f[k];
+      v[k] = vel[3 * i + k];
+      if (dt_kick > 0.0) v[k] += h * (double)f[k];   // not with 0 times a force that may not be finite
       v2 += v[k] * v[k];
     }
     ke = (0.5 * kKinetic) * mass[i] * v2;

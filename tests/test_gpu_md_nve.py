@@ -90,3 +90,23 @@ def test_nve_zero_steps_and_bad_arguments(ctx):
         ctx.md_nve(p, d(v), d(m), box, P2, 0.0, 5)
     with pytest.raises(binding.TersoffError):
         ctx.md_nve(p, p, d(m), box, P2, 1.0, 5)
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("nsteps", [0, 1])
+def test_nve_first_evaluation_kicks_nothing(ctx, precision, nsteps):
+    """The first evaluation is not a kick: with forces that are not finite (parameters whose pair functions overflow) the
+    kinetic energy before the first step is that of the given velocities, and with no steps they stay as they are."""
+    pos, box, m, v = _system((3, 3, 3), 300.0, 6)
+    p, x = torch.tensor(pos, device="cuda"), torch.tensor(v, device="cuda")
+    x[0, 0] = -0.0
+    want = omd.kinetic_energy(x.cpu().numpy(), m)
+    before = x.clone()
+    params = [1e300, 1000.0, 3.0, 0.28, 0.6, -0.64]
+    Ep, Ek, F, W = ctx.md_nve(p, x, torch.tensor(m, device="cuda"), box, params, 1.0, nsteps, precision=precision)
+    torch.cuda.synchronize()
+    assert nsteps or not torch.isfinite(F).all()
+    assert abs(float(Ek[0]) - want) <= 1e-12 * want
+    if nsteps == 0:
+        assert torch.equal(x.view(torch.int64), before.view(torch.int64))
+    ctx.get_status()
