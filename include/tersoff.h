@@ -128,7 +128,8 @@ int tersoff_build_info(tersoff_ctx *ctx, int64_t *ntot, int64_t *nbonds, int32_t
  *  F         device [P][Ntot][3] float or double (see precision) -- may be NULL
  *  W         device [P][C][6] double, total virial (eV)          -- may be NULL
  * Atoms with more than 8 neighbours are not supported by the evaluation kernels: the build reports
- * them and this call returns TERSOFF_E_UNSUPPORTED. */
+ * them and this call returns TERSOFF_E_UNSUPPORTED. A call that returns an error of the build leaves
+ * E, F and W as they were. */
 int tersoff_eval(tersoff_ctx *ctx, const double *params, int32_t P, int32_t precision, double *E,
                  void *F, double *W, tersoff_stream stream);
 

@@ -102,6 +102,7 @@ cudaError_t launch_batch(const Ctx &ctx, const BatchPlan &plan, const double *pa
   bp.F = out.F;
   bp.f_ld = out.f_ld;
   bp.aw = out.aw;
+  bp.build_status = out.build_status;
   bp.W = out.W;
   bp.tE = out.tE;
   bp.tW = out.tW;

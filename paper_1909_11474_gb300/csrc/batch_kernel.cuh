@@ -536,6 +536,7 @@ struct BatchParams {
   double *part;                    // [P][C][3]: FP64 residual terms e, v, f of every (p, c) (fitness)
   double *dpart;                   // [C][3]: FP64 target-norm terms of every configuration (fitness)
   unsigned *status;
+  const unsigned *build_status;    // evaluation queued ahead of a rebuild's check: that build's errors, or null
 };
 
 // Shared memory of one CTA (R = float or double, R4 its 4-vector):
@@ -1087,6 +1088,7 @@ __global__ void __launch_bounds__(NW * kWarp, MINB) batch_kernel(const BatchPara
     // item whose configuration changed is skipped (the host launches again on the new schedule).
     // Every warp checks the records of all ranks of the item, one a lane, so a cluster decides alike (with the
     // records in turn, each a chain of two loads, this took 13 of 101 us for 100 cells of 64 to 512 atoms x 200 sets).
+    // An evaluation so queued writes nothing at all after a build that failed (lane 31, which has no record to check).
     {
       bool match = true;
       if (lane < (int)ncta) {
@@ -1097,6 +1099,8 @@ __global__ void __launch_bounds__(NW * kWarp, MINB) batch_kernel(const BatchPara
                   a.poff[l] + pair_slots(ml) == q.Q0 + q.nq;
         }
       }
+      static_assert(kMaxCluster < 32, "a lane beside the records");
+      if (!FIT && lane == 31 && a.build_status) match = *a.build_status == 0u;
       match = __all_sync(0xffffffffu, match);
       if (!match) {
         // every warp of every rank comes here; none may still have to read s_item when the next item is claimed

@@ -354,8 +354,9 @@ int tersoff_create(tersoff_ctx **out, int device) {
   tersoff_ctx *ctx = new tersoff_ctx();
   ctx->c.device = device;
   cudaDeviceGetAttribute(&ctx->c.nsm, cudaDevAttrMultiProcessorCount, device);
-  if (ctx->c.status.ensure(sizeof(unsigned)) != cudaSuccess ||
-      cudaMemset(ctx->c.status.p, 0, sizeof(unsigned)) != cudaSuccess) {
+  // two words: the context's status, then the last neighbour build's own
+  if (ctx->c.status.ensure(2 * sizeof(unsigned)) != cudaSuccess ||
+      cudaMemset(ctx->c.status.p, 0, 2 * sizeof(unsigned)) != cudaSuccess) {
     delete ctx;
     return TERSOFF_E_CUDA;
   }
@@ -551,7 +552,7 @@ int tersoff_build_neighbors(tersoff_ctx *ctx, const tersoff_configs *cfg, double
   }
   int nat_max = 1;
   for (int k = 0; k < C; ++k) nat_max = std::max(nat_max, cfg->atom_off[k + 1] - cfg->atom_off[k]);
-  TSF_CUDA(cudaMemsetAsync(c.status.p, 0, sizeof(unsigned), s));
+  TSF_CUDA(cudaMemsetAsync(c.status.p, 0, 2 * sizeof(unsigned), s));   // status and build status
   unsigned *st = c.status.as<unsigned>();
   tsf::BuildLaunch L = {};
   L.C = C;
@@ -576,6 +577,7 @@ int tersoff_build_neighbors(tersoff_ctx *ctx, const tersoff_configs *cfg, double
   L.ameta = c.ameta.as<int>();
   L.arev = c.arev.as<int4>();
   L.status = st;
+  L.build_status = st + 1;
   L.h_cnt = hp;
   L.h_flag = hp + tsf::build_flags_at(N, C);
   L.nat_max = nat_max;
@@ -619,9 +621,10 @@ int tersoff_build_info(tersoff_ctx *ctx, int64_t *ntot, int64_t *nbonds, int32_t
   return TERSOFF_OK;
 }
 
-// Queues one evaluation on the current schedule.
+// Queues one evaluation on the current schedule; ahead: before the host has checked the build, whose errors the kernels
+// then look at themselves.
 static int queue_eval(tersoff_ctx *ctx, const double *params, int32_t P, int32_t precision, double *E, void *F,
-                      double *W, tersoff_stream stream) {
+                      double *W, bool ahead, tersoff_stream stream) {
   Ctx &c = ctx->c;
   cudaSetDevice(c.device);
   int rc = build_plan(ctx, precision);
@@ -636,6 +639,7 @@ static int queue_eval(tersoff_ctx *ctx, const double *params, int32_t P, int32_t
   o.F = F;
   o.W = W;
   o.consts = c.work.p;
+  if (ahead) o.build_status = c.status.as<unsigned>() + 1;
   TSF_CUDA(tsf::launch_batch(c, precision == 64 ? c.plan64 : c.plan32, params, P, tsf::kModeEval, o, S(stream)));
   return TERSOFF_OK;
 }
@@ -671,7 +675,7 @@ int tersoff_eval(tersoff_ctx *ctx, const double *params, int32_t P, int32_t prec
     if (int rc = may_speculate(ctx, precision, S(stream), &ahead)) return rc;
   if (ahead) {
     const uint64_t gen = c.plan32.gen;
-    if (int rc = queue_eval(ctx, params, P, precision, E, F, W, stream)) return rc;
+    if (int rc = queue_eval(ctx, params, P, precision, E, F, W, true, stream)) return rc;
     if (int rc = tsf::finish_build(ctx)) return rc;
     if (c.plan32.gen == gen && !c.plan32.buckets.empty()) return TERSOFF_OK;
     TSF_CUDA(cudaMemsetAsync(c.status.p, 0, sizeof(unsigned), S(stream)));
@@ -681,7 +685,7 @@ int tersoff_eval(tersoff_ctx *ctx, const double *params, int32_t P, int32_t prec
   if (!params || P < 1) return fail(ctx, TERSOFF_E_ARG, "need params and P >= 1%s");
   if (precision != 32 && precision != 64) return fail(ctx, TERSOFF_E_ARG, "precision must be 32 or 64%s");
   if (c.max_m > 8) return fail(ctx, TERSOFF_E_UNSUPPORTED, "an atom has more than 8 neighbours%s");
-  return queue_eval(ctx, params, P, precision, E, F, W, stream);
+  return queue_eval(ctx, params, P, precision, E, F, W, false, stream);
 }
 
 int tersoff_fitness(tersoff_ctx *ctx, const double *params, int32_t P, const tersoff_targets *tg,

@@ -239,7 +239,7 @@ struct BuildLaunch {
   float *gcos;
   int *ameta;
   int4 *arev;
-  unsigned *status;                // the context's status word
+  unsigned *status, *build_status; // the context's status word and the build's own
   int *h_cnt, *h_flag;             // pinned host memory the kernel writes (BuildParams)
   int nat_max;    // largest configuration (atoms)
 };
@@ -265,6 +265,7 @@ struct BatchOut {
   bool pdl = false;   // launch the batched kernels with programmatic stream serialization
   int64_t wait_spins = -1;   // polls of the staging wait before it gives up (negative: built-in bound)
   int form = 0;       // 0: minimal (6 parameters), 1: Tersoff form (9 parameters, Eq. 8, free S)
+  const unsigned *build_status = nullptr;   // evaluation queued ahead of a rebuild's check: the build's status word
   int64_t f_ld = 0;   // gradient: F receives v = 2 (F - F*) as [Ntot][3][f_ld], parameter sets fastest
   float *aw = nullptr;   // gradient: weights a_e, a_k [C][7][f_ld]
 };

@@ -198,7 +198,7 @@ struct BuildParams {
   float *gcos;
   int *ameta;                      // [Ntot]: bonds kept (min(cnt, M)) | (some bond beyond R1) << 16
   int4 *arev;                      // [Ntot]: configuration-local reverse bonds of the first 8 bonds, 16 bits each
-  unsigned *status;                // the context's status word
+  unsigned *status, *build_status; // the context's status word and this build's own
   int *h_cnt, *h_flag;             // pinned host memory: bonds kept of every atom; [0] set on non-finite input, [1] on an overflow
   int nat_max;                     // largest configuration of the launch (shared-memory layout)
   int lists_in_smem;               // the lists and unit vectors fit in shared memory
@@ -209,6 +209,7 @@ struct BuildParams {
 
 __device__ __forceinline__ void build_flag(const BuildParams &a, unsigned bit) {
   set_status(a.status, bit);
+  set_status(a.build_status, bit);
   a.h_flag[bit == TERSOFF_STATUS_NONFINITE ? 0 : 1] = 1;
 }
 
@@ -752,6 +753,7 @@ cudaError_t launch_build_batch(const BuildLaunch &L, cudaStream_t s) {
   a.ameta = L.ameta;
   a.arev = L.arev;
   a.status = L.status;
+  a.build_status = L.build_status;
   a.h_cnt = L.h_cnt;
   a.h_flag = L.h_flag;
   a.nat_max = std::max(1, L.nat_max);

@@ -624,3 +624,40 @@ def test_rebuild_with_a_long_list_and_equal_totals(tile, P):
     for x, y in zip(c.fitness(params, t), want):
         assert np.allclose(x.cpu(), y, rtol=1e-6)
     assert c.get_status() == 0
+
+
+@pytest.mark.parametrize("change", ["overflow", "nonfinite"])
+@pytest.mark.parametrize("C,reps", [(1, (2, 2, 2)), (6, (2, 2, 2)), (3, (4, 4, 2))])
+def test_failed_rebuild_leaves_the_outputs_of_an_evaluation(change, C, reps):
+    """The evaluation that returns a rebuild's error writes nothing: E, F and W keep what they held."""
+    from paper_1909_11474_gb300 import binding
+    rng = np.random.default_rng(3)
+    cs = I.make_cells(rng, C, lambda: reps, lambda: I.random_strain(rng, 0.01), lambda: 0.05, lambda: 0)
+    P = 9
+    params = torch.tensor(I.population(rng, P)[0], device="cuda")
+    c = binding.Context(0)
+    _build(c, cs)
+    c.eval(params)
+    pos2 = cs.pos.copy()
+    a0 = cs.atom_off[C - 1]
+    if change == "overflow":                  # 33 atoms within a sphere of radius 0.8
+        d = np.random.default_rng(1).normal(size=(33, 3))
+        pos2[a0:a0 + 33] = pos2[a0] + 0.8 * d / np.linalg.norm(d, axis=1)[:, None]
+    else:
+        pos2[a0, 1] = np.nan
+    p2, b2 = torch.tensor(pos2, device="cuda"), torch.tensor(cs.box, device="cuda")
+    out = [torch.full(s, 7.0, dtype=t, device="cuda") for s, t in
+           (((P, C), torch.float64), ((P, cs.Ntot, 3), torch.float32), ((P, C, 6), torch.float64))]
+    c.build_neighbors(cs.atom_off, p2, b2, 2.8, 3.2, 16)
+    rc = c.lib.tersoff_eval(c.h, params.data_ptr(), P, 32, *(x.data_ptr() for x in out), binding._stream(None))
+    torch.cuda.synchronize()
+    assert rc == (binding.E_NBR_OVERFLOW if change == "overflow" else binding.E_NONFINITE)
+    for x in out:
+        assert (x == 7.0).all()
+    c.get_status()
+    _build(c, cs)                             # and a valid rebuild evaluates again
+    fresh = binding.Context(0)
+    _build(fresh, cs)
+    for x, y in zip(c.eval(params), fresh.eval(params)):
+        assert torch.equal(x, y)
+    assert c.get_status() == 0
