@@ -303,14 +303,15 @@ cudaError_t launch_fitness_finalize(int P, int C, const double *part, const doub
   return e;
 }
 
-// Module loading of every kernel the minimal-form fitness path launches.
-cudaError_t preload_fitness_kernels() {
+// Module loading of every kernel that the minimal form's fitness and evaluation launch.
+cudaError_t preload_batch_kernels() {
   cudaFuncAttributes fa;
   cudaError_t e = cudaFuncGetAttributes(&fa, prep_kernel<float>);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, prep_kernel<double>);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fitness_finalize_kernel);
   if (e == cudaSuccess) e = preload_fitness32();
-  if (e == cudaSuccess) e = preload_fitness64();
+  if (e == cudaSuccess) e = preload_eval32();
+  if (e == cudaSuccess) e = preload_batch64();
   if (e == cudaSuccess) e = preload_geometry64_kernels();
   return e;
 }

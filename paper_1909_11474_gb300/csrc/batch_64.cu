@@ -6,9 +6,9 @@ namespace tsf {
 template cudaError_t launch_bucket<double, false, true>(const BatchParams &, const Bucket &, bool, cudaStream_t);
 template cudaError_t launch_bucket<double, false, false>(const BatchParams &, const Bucket &, bool, cudaStream_t);
 
-cudaError_t preload_fitness64() {
-  cudaError_t e = touch_variant<kPT64, 8, false, 1, double, kNW>();
-  if (e == cudaSuccess) e = touch_variant<kPT64, 8, true, 1, double, kNW>();
+cudaError_t preload_batch64() {
+  cudaError_t e = touch_variants64<true>();
+  if (e == cudaSuccess) e = touch_variants64<false>();
   return e;
 }
 

@@ -5,6 +5,8 @@ namespace tsf {
 
 template cudaError_t launch_bucket<float, false, false>(const BatchParams &, const Bucket &, bool, cudaStream_t);
 
+cudaError_t preload_eval32() { return touch_variants32<false>(); }
+
 TSF_DEBUG_TAKE(debug_take_eval32)
 
 }  // namespace tsf

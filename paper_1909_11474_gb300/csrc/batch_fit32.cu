@@ -6,14 +6,9 @@ namespace tsf {
 template cudaError_t launch_bucket<float, false, true>(const BatchParams &, const Bucket &, bool, cudaStream_t);
 
 cudaError_t preload_fitness32() {
-  cudaError_t e = touch_variant<16, 4, false, 3, float, kNW>();
-  if (e == cudaSuccess) e = touch_variant<kPT, 4, false, 2, float, 12>();
-  if (e == cudaSuccess) e = touch_variant<kPT, 4, false, 2, float, kNW>();
-  if (e == cudaSuccess) e = touch_variant<kPT, 6, false, 2, float, kNW>();
-  if (e == cudaSuccess) e = touch_variant<kPT, 8, false, 2, float, kNW>();
-  if (e == cudaSuccess) e = touch_variant<kPT, 4, true, 2, float, kNW>();
-  if (e == cudaSuccess) e = touch_variant<kPT, 6, true, 2, float, kNW>();
-  if (e == cudaSuccess) e = touch_variant<kPT, 8, true, 2, float, kNW>();
+  cudaError_t e = touch_variant<16, 4, false, 3, float, kNW, true>();
+  if (e == cudaSuccess) e = touch_variant<kPT, 4, false, 2, float, 12, true>();
+  if (e == cudaSuccess) e = touch_variants32<true>();
   return e;
 }
 

@@ -121,12 +121,29 @@ cudaError_t launch_bucket(const BatchParams &bp, const Bucket &b, bool pdl, cuda
   }
 }
 
-// Force the module loading of every fitness kernel of one precision in the minimal form (with lazy loading
-// the driver would load each on its first launch, allocating device memory for its code then).
-template <int PTV, int MMAX, bool CLUSTER, int MINB, typename R, int NW>
+// Force the module loading of every kernel of one precision in the minimal form, for the fitness (FIT) or for
+// evaluation and gradient (with lazy loading the driver would load each on its first launch, allocating device memory
+// for its code then).
+template <int PTV, int MMAX, bool CLUSTER, int MINB, typename R, int NW, bool FIT>
 inline cudaError_t touch_variant() {
   cudaFuncAttributes fa;
-  return cudaFuncGetAttributes(&fa, batch_kernel<PTV, MMAX, CLUSTER, MINB, R, NW, false, true>);
+  return cudaFuncGetAttributes(&fa, batch_kernel<PTV, MMAX, CLUSTER, MINB, R, NW, false, FIT>);
+}
+template <bool FIT>
+inline cudaError_t touch_variants32() {
+  cudaError_t e = touch_variant<kPT, 4, false, 2, float, kNW, FIT>();
+  if (e == cudaSuccess) e = touch_variant<kPT, 6, false, 2, float, kNW, FIT>();
+  if (e == cudaSuccess) e = touch_variant<kPT, 8, false, 2, float, kNW, FIT>();
+  if (e == cudaSuccess) e = touch_variant<kPT, 4, true, 2, float, kNW, FIT>();
+  if (e == cudaSuccess) e = touch_variant<kPT, 6, true, 2, float, kNW, FIT>();
+  if (e == cudaSuccess) e = touch_variant<kPT, 8, true, 2, float, kNW, FIT>();
+  return e;
+}
+template <bool FIT>
+inline cudaError_t touch_variants64() {
+  cudaError_t e = touch_variant<kPT64, 8, false, 1, double, kNW, FIT>();
+  if (e == cudaSuccess) e = touch_variant<kPT64, 8, true, 1, double, kNW, FIT>();
+  return e;
 }
 #ifdef TSF_DEBUG_BOUNDS
 // Reads and clears a translation unit's bounds record (tersoff_debug_bounds).
@@ -143,6 +160,7 @@ cudaError_t debug_take_fit32(unsigned *), debug_take_eval32(unsigned *), debug_t
 #define TSF_DEBUG_TAKE(name)
 #endif
 cudaError_t preload_fitness32();   // batch_fit32.cu
-cudaError_t preload_fitness64();   // batch_64.cu
+cudaError_t preload_eval32();      // batch_eval32.cu
+cudaError_t preload_batch64();     // batch_64.cu
 
 }  // namespace tsf

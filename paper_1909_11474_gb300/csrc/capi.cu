@@ -536,10 +536,10 @@ int tersoff_build_neighbors(tersoff_ctx *ctx, const tersoff_configs *cfg, double
   TSF_CUDA(c.gA32.ensure(bond_cap * sizeof(float4)));
   TSF_CUDA(c.gB32.ensure(bond_cap * sizeof(float4)));
   TSF_CUDA(c.gcos32.ensure(slot_cap * sizeof(float)));
-  // everything the later calls of this build need is allocated here, so that those calls (the
-  // allocation-free fitness among them) allocate nothing: the FP64 geometry records (computed on the
-  // first FP64 use), the work-schedule records of both precisions, the side streams, and the code of
-  // the fitness kernels (loaded up front instead of lazily on their first launch)
+  // what later calls need of this build is allocated here: the FP64 geometry records (computed on the first FP64 use),
+  // the work-schedule records of both precisions, the side streams, and the code of the minimal form's fitness and
+  // evaluation kernels (loaded up front instead of lazily on their first launch). The allocation-free fitness then
+  // allocates nothing; the other calls grow workspaces that depend on the number of parameter sets on first use
   TSF_CUDA(c.gA64.ensure(bond_cap * sizeof(tsf::dvec4)));
   TSF_CUDA(c.gB64.ensure(bond_cap * sizeof(tsf::dvec4)));
   TSF_CUDA(c.gcos64.ensure(slot_cap * sizeof(double)));
@@ -547,7 +547,7 @@ int tersoff_build_neighbors(tersoff_ctx *ctx, const tersoff_configs *cfg, double
   TSF_CUDA(c.plan64.items.ensure((size_t)C * tsf::kMaxClusterCtas * sizeof(tsf::CtaRec)));
   TSF_CUDA(tsf::ensure_side_streams(c));
   if (!c.preloaded) {
-    TSF_CUDA(tsf::preload_fitness_kernels());
+    TSF_CUDA(tsf::preload_batch_kernels());
     c.preloaded = true;
   }
   int nat_max = 1;

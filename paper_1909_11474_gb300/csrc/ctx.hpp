@@ -274,10 +274,10 @@ cudaError_t launch_batch(const Ctx &ctx, const BatchPlan &plan, const double *pa
                          int mode, const BatchOut &out, cudaStream_t s);
 cudaError_t autotune_batch(const Ctx &ctx, BatchPlan &plan, const double *params, int P, int mode,
                            const BatchOut &out, int reps, cudaStream_t s, float *best_ms, int *tried);
-// Side streams of the launch buckets, and the module loading of every kernel a fitness call can launch
-// (so that later calls neither create resources nor load code on the device).
+// Side streams of the launch buckets, and the module loading of every kernel that a fitness or
+// evaluation call can launch in the minimal form (so that later calls neither create resources nor load code on the device).
 cudaError_t ensure_side_streams(const Ctx &ctx);
-cudaError_t preload_fitness_kernels();
+cudaError_t preload_batch_kernels();
 cudaError_t preload_geometry64_kernels();   // neighbors.cu
 cudaError_t launch_fitness_finalize(int P, int C, const double *part, const double *dpart,
                                     double we, double wv, double wf, double *Z, double *Zq, double *S, bool pdl,

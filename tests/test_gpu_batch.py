@@ -661,3 +661,42 @@ def test_failed_rebuild_leaves_the_outputs_of_an_evaluation(change, C, reps):
     for x, y in zip(c.eval(params), fresh.eval(params)):
         assert torch.equal(x, y)
     assert c.get_status() == 0
+
+
+PRELOAD = """
+import numpy as np, torch
+from paper_1909_11474_gb300 import binding, inputs as I
+rng = np.random.default_rng(3)
+cs = I.make_cells(rng, 4, lambda: (2, 2, 2), lambda: I.random_strain(rng, 0.02), lambda: 0.1, lambda: 0)
+ctx = binding.Context(0)
+pos, box = torch.tensor(cs.pos, device="cuda"), torch.tensor(cs.box, device="cuda")
+params = torch.tensor(I.population(rng, 21)[0], device="cuda")
+t = {"E": torch.full((4,), -4.6), "W": torch.zeros((4, 6)), "F": torch.zeros((cs.Ntot, 3))}
+t = {k: v.double().cuda() for k, v in t.items()} | {"mask": torch.full((4,), 7, dtype=torch.uint8, device="cuda")}
+out = [torch.empty(s, dtype=d, device="cuda") for s, d in
+       (((21, 4), torch.float64), ((21, cs.Ntot, 3), torch.float64), ((21, 4, 6), torch.float64))]
+ctx.build_neighbors(cs.atom_off, pos, box, 2.8, 3.2, 16)
+for precision in (32, 64):
+    ctx.fitness(params, t, precision=precision)       # the workspaces that fitness and evaluation share
+torch.cuda.synchronize()
+free = [torch.cuda.mem_get_info()[0]]
+for precision in (32, 64):
+    rc = ctx.lib.tersoff_eval(ctx.h, params.data_ptr(), 21, precision, *(x.data_ptr() for x in out), binding._stream(None))
+    torch.cuda.synchronize()
+    free.append(torch.cuda.mem_get_info()[0])
+    assert rc == 0
+print(*free)
+"""
+
+
+def test_first_evaluation_after_a_build_loads_no_code():
+    """The build loads the evaluation kernels of both precisions too: free device memory does not change across a process's
+    first evaluations. (In a process of its own, where no other test has loaded them.)"""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", PRELOAD], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
+    free = r.stdout.split()[-3:]
+    assert free[0] == free[1] == free[2], free
