@@ -238,7 +238,8 @@ int tersoff_ga_step(int32_t P, int32_t n_genes, int32_t n_par, double rate, cons
  *  closed-form derivatives per atom; populations whose workspace would exceed 1 GiB in blocks).
  *  loss TERSOFF_LOSS_SQ or TERSOFF_LOSS_Z (the latter has a zero gradient term where S_q = 0);
  *  L device [P] double; dL device [P][6] ([P][9] in the Tersoff form) double. FP32 per-pair arithmetic with FP64 accumulation of
- *  the residual sums and of the gradient. Forces enter through the directional derivative
+ *  the residual sums and of the gradient. After a staging wait that gives up (tersoff_set_wait_limit) L and dL are
+ *  undefined. Forces enter through the directional derivative
  *  sum_i v_i . dF_i/dx = -d/dx [ sum_i sum_j (v_j - v_i) . dU_i/dd_ij ] with v_i = dL/dF_i. */
 int tersoff_param_grad(tersoff_ctx *ctx, const double *params, int32_t P, const tersoff_targets *tg,
                        const double *w, int32_t loss, double *L, double *dL, tersoff_stream stream);
@@ -300,7 +301,8 @@ int tersoff_set_launch_mode(tersoff_ctx *ctx, int32_t mode);
 
 /* Bound of the device-side wait of this context's later calls; the paper has no counterpart. One kernel
  * waits on other work: the batched kernel waits for the bulk copies that stage a configuration's
- * geometry in shared memory (tersoff_eval, tersoff_fitness, tersoff_fitness_static, tersoff_autotune).
+ * geometry in shared memory (tersoff_eval, tersoff_fitness, tersoff_fitness_static, tersoff_param_grad,
+ * tersoff_autotune).
  * The wait polls at most `spins` times (0: it gives up at once unless the copies have already landed);
  * a negative value restores the built-in bound (2^22 polls, far beyond any wait that can end). A wait
  * that gives up sets TERSOFF_STATUS_TIMEOUT in the status word, and its CTA stops without its results

@@ -50,3 +50,21 @@ def test_staging_wait_that_gives_up_reports_a_timeout(graphs):
     E1, F1, W1 = (x.cpu().numpy() for x in ctx.eval(params))
     assert ctx.get_status() == 0
     assert np.array_equal(Z1, Z0) and np.array_equal(E1, E0) and np.array_equal(F1, F0) and np.array_equal(W1, W0)
+
+
+def test_gradient_takes_the_bounded_wait():
+    """tersoff_param_grad runs the batched kernel too: its wait gives up and is reported alike, and the next call with the
+    built-in bound gives the results from before."""
+    from paper_1909_11474_gb300 import binding
+    ctx = binding.Context(0)
+    params, tg = _fitness_setup(ctx)
+    want = [x.cpu().numpy() for x in ctx.param_grad(params, tg)]
+    assert ctx.get_status() == 0
+    ctx.set_wait_limit(0)
+    ctx.param_grad(params, tg)
+    assert ctx.get_status() & binding.STATUS_TIMEOUT
+    ctx.set_wait_limit(-1)
+    got = [x.cpu().numpy() for x in ctx.param_grad(params, tg)]
+    assert ctx.get_status() == 0
+    for a, b in zip(got, want):
+        assert np.array_equal(a, b)
