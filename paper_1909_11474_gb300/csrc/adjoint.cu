@@ -556,9 +556,9 @@ static cudaError_t launch_tangent(const TangentParams &a, dim3 grid, bool pdl, c
 }
 
 // Parameter sets handled by one launch sequence: all of them, or blocks of a multiple of 32 so that v stays
-// within 1 GiB.
+// within 1 GiB and the tiles (32 wide for blocks of that size) within a grid's 65,535 rows.
 int grad_block(int64_t Ntot, int P) {
-  const int64_t most = std::max<int64_t>(1, (int64_t{1} << 30) / (Ntot * 12 * 32)) * 32;
+  const int64_t most = std::min<int64_t>(65535, std::max<int64_t>(1, (int64_t{1} << 30) / (Ntot * 12 * 32))) * 32;
   return (int)std::min<int64_t>(P, most);
 }
 GradPlan grad_plan(const Ctx &ctx, int P) {

@@ -237,3 +237,22 @@ def test_param_grad_in_blocks_of_parameter_sets():
         L1, dL1 = ctx.param_grad(x[a:b].contiguous(), tg, w=WTS, loss=0)
         assert torch.allclose(L[a:b], L1, rtol=1e-6, atol=0)
         assert ((dL[a:b] - dL1).abs() <= GRAD_TOL * dL1.abs().amax(1, keepdim=True)).all()
+
+
+def test_param_grad_of_more_sets_than_a_grid_has_rows():
+    """2,097,216 sets on one 8-atom cell (the tiles of a launch are its grid's rows, at most 65,535): 64 sets repeated, so
+    every repetition has the gradient of the first."""
+    from paper_1909_11474_gb300 import binding
+    rng = np.random.default_rng(4)
+    cs = I.make_cells(rng, 1, lambda: (1, 1, 1), lambda: I.random_strain(rng, 0.02), lambda: 0.1, lambda: 0)
+    t = {"E": np.full(1, -4.6), "W": np.zeros((1, 6)), "F": np.zeros((cs.Ntot, 3)), "mask": np.full(1, 7, np.uint8)}
+    ctx = binding.Context(0)
+    pos, box = to_device(cs)
+    ctx.build_neighbors(cs.atom_off, pos, box, 2.8, 3.2, 16)
+    n = 32769
+    params = torch.tensor(I.population(rng, 64)[0], device="cuda").repeat(n, 1)
+    L, dL = ctx.param_grad(params, targets_to_device(t))
+    L, dL = L.view(n, 64), dL.view(n, 64, 6)
+    assert torch.isfinite(dL).all() and ctx.get_status() == 0
+    assert ((L - L[0]).abs() <= 1e-6 * L[0].abs()).all()
+    assert ((dL - dL[0]).abs() <= 1e-6 * dL[0].abs().amax()).all()
