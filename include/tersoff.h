@@ -197,7 +197,8 @@ int tersoff_autotune(tersoff_ctx *ctx, const double *params, int32_t P, const te
 /* Set the batched fitness schedule by hand (what tersoff_autotune would choose); the paper has no
  * counterpart. For every launch bucket of `precision` and calls with this P: tile = 32 parameter
  * sets per tile (one atom per warp), or 16 (two atoms per warp, three CTAs per SM; only for the FP32
- * single-CTA variant of up to 4 neighbours, others keep 32); warps = 8 or 12 per CTA (12: 32-wide
+ * single-CTA variant of up to 4 neighbours, others keep 32; the FP64 kernels have tiles of 8, which 8
+ * and 32 stand for); warps = 8 or 12 per CTA (12: 32-wide
  * tiles of that same variant only, at most 80 registers, two CTAs per SM); items_per_config >= 1 work items per
  * configuration (the parameter tiles split into that many chunks, capped at the tile count);
  * narrow = 1 lets a partly filled last tile run with more atoms per warp. Kept until a rebuild

@@ -763,9 +763,10 @@ int tersoff_set_schedule(tersoff_ctx *ctx, int32_t precision, int32_t P, int32_t
   Ctx &c = ctx->c;
   if (int rc = tsf::finish_build(ctx)) return rc;
   if (precision != 32 && precision != 64) return fail(ctx, TERSOFF_E_ARG, "precision must be 32 or 64%s");
-  if (P < 1 || items_per_config < 1 || (tile != 32 && tile != 16) || (warps != 8 && warps != 12) ||
+  // 32 stands for the precision's own width too, which tersoff_schedule_info reports
+  if (P < 1 || items_per_config < 1 || (tile != 32 && tile != 16 && tile != tsf::batch_param_tile(precision)) || (warps != 8 && warps != 12) ||
       (narrow != 0 && narrow != 1))
-    return fail(ctx, TERSOFF_E_ARG, "need P >= 1, tile 32 or 16, warps 8 or 12, items_per_config >= 1, narrow 0 or 1%s");
+    return fail(ctx, TERSOFF_E_ARG, "need P >= 1, tile 32 or 16 (FP64: or 8), warps 8 or 12, items_per_config >= 1, narrow 0 or 1%s");
   if (c.max_m > 8) return fail(ctx, TERSOFF_E_UNSUPPORTED, "an atom has more than 8 neighbours%s");
   int rc = build_plan(ctx, precision);
   if (rc) return rc;

@@ -700,3 +700,27 @@ def test_first_evaluation_after_a_build_loads_no_code():
     assert r.returncode == 0, r.stderr
     free = r.stdout.split()[-3:]
     assert free[0] == free[1] == free[2], free
+
+
+@pytest.mark.parametrize("precision", [32, 64])
+def test_schedule_read_back_can_be_set(ctx, precision):
+    """What schedule_info reports of a tuned schedule is what set_schedule takes (a program that keeps the schedules it has
+    tuned), and the results are the tuned ones."""
+    w = I.workload_ga_batch(P=45, C=5)
+    cs = w["configs"]
+    t = {"E": np.full(cs.C, -4.6), "W": np.zeros((cs.C, 6)), "F": np.zeros((cs.Ntot, 3)),
+         "mask": np.full(cs.C, 7, np.uint8)}
+    params, tg = torch.tensor(w["params"], device="cuda"), targets_to_device(t)
+    _build(ctx, cs)
+    ctx.autotune(params, tg, precision=precision, reps=1)
+    want = ctx.fitness(params, tg, precision=precision)
+    info = ctx.schedule_info(precision)
+    _build(ctx, I.workload_ga_batch(P=45, C=4)["configs"])
+    _build(ctx, cs)
+    b = info[0]
+    ctx.set_schedule(b["tuned_P"], tile=b["tile"], items_per_config=b["items_per_config"], narrow=bool(b["narrow"]),
+                     precision=precision, warps=b["warps"])
+    assert ctx.schedule_info(precision) == info
+    for x, y in zip(ctx.fitness(params, tg, precision=precision), want):
+        assert torch.equal(x, y)
+    assert ctx.get_status() == 0
