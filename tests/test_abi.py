@@ -55,3 +55,19 @@ def test_build_watches_every_included_file():
         path = os.path.join(build.CSRC, name)
         for inc in re.findall(r'^\s*#include "([^"]+)"', open(path).read(), re.M):
             assert os.path.realpath(os.path.join(build.CSRC, inc)) in deps, f"{name} includes {inc}"
+
+
+def test_current_stream_without_pytorchs_private_calls(monkeypatch):
+    """The current stream's handle comes the public way where PyTorch has no private calls for it."""
+    import types
+
+    import torch
+
+    from paper_1909_11474_gb300 import binding
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=1234))
+    monkeypatch.setattr(binding, "_raw_device", lambda: 3)
+    monkeypatch.setattr(binding, "_raw_stream", lambda device: 100 + device)
+    assert binding._stream(None) == 103
+    monkeypatch.setattr(binding, "_raw_stream", None)
+    assert binding._stream(None) == 1234
