@@ -65,7 +65,8 @@ __device__ __forceinline__ double scale2(double x, int k) {
   return fx_from_bits(fx_bits(x) + ((uint64_t)(int64_t)k << 52));
 }
 
-// 1/x to within an ulp, from the FP32 reciprocal (e = 1 - x y0 is below 2^-22, the cubic step leaves e^3).
+// 1/x to within 0.5002 ulp (a divide: 0.5), from the FP32 reciprocal (e = 1 - x y0 is exact and below 2^-22, the cubic
+// step leaves e^3, and only its last operation rounds).
 __device__ __forceinline__ double rcp64(double x) {
   const int e = (int)((fx_bits(x) >> 52) & 0x7ffu) - 1023;
   if (e < -100 || e > 100) return 1.0 / x;
@@ -74,7 +75,7 @@ __device__ __forceinline__ double rcp64(double x) {
   return __fma_rn(y0, __fma_rn(d, d, d), y0);
 }
 
-// 1/sqrt(x) to within an ulp, likewise (third-order step).
+// 1/sqrt(x) to within 1.0002 ulp (the reciprocal of a rounded square root: 1.5), likewise; here x y0 is rounded.
 __device__ __forceinline__ double rsqrt64(double x) {
   const int e = (int)((fx_bits(x) >> 52) & 0x7ffu) - 1023;
   if (e < -100 || e > 100) return rsqrt(x);

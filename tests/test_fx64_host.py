@@ -132,3 +132,24 @@ def test_fixed_point_bond_functions_at_the_ends_of_their_ranges(tmp_path):
     subprocess.run([cxx, "-O2", "-std=c++17", "-I", CSRC, str(src), "-o", str(exe)], check=True)
     taken, wrong = (int(x) for x in subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split())
     assert taken > 200000 and wrong == 0, (taken, wrong)
+
+
+def test_fixed_point_tables_recomputed():
+    """Every entry of fx64_tables.inc from its definition, in 60-digit decimal arithmetic, and the bound that the
+    logarithm's polynomial rests on: |m c_j - 1| < 2^-8.6 over the interval of j."""
+    import re
+    from decimal import ROUND_HALF_EVEN, Decimal, getcontext
+    getcontext().prec = 60
+    body = open(os.path.join(CSRC, "fx64_tables.inc")).read().split("= {", 1)[1]
+    exp2, log_inv, inv = ([int(x, 0) for x in re.findall(r"0x[0-9a-f]+|\d+", part.replace("ull", ""))]
+                          for part in re.findall(r"\{([^{}]*)\}", body))
+    assert len(exp2) == len(log_inv) == len(inv) == 256
+    ln2 = Decimal(2).ln()
+    nearest = lambda x: int(x.to_integral_value(rounding=ROUND_HALF_EVEN))   # noqa: E731
+    for j in range(256):
+        assert exp2[j] == nearest((ln2 * j / 256).exp() * 2 ** 63)
+        assert inv[j] == nearest(Decimal(2 ** 11) / (1 + (Decimal(j) + Decimal("0.5")) / 256))
+        c = Decimal(inv[j]) / 2 ** 11
+        assert log_inv[j] == nearest(-c.ln() / ln2 * 2 ** 62)
+        for m in (1 + Decimal(j) / 256, 1 + Decimal(j + 1) / 256):
+            assert abs(m * c - 1) < Decimal(2) ** Decimal("-8.6")
