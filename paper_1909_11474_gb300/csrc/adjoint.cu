@@ -58,7 +58,7 @@ struct TangentParams {
 template <bool GEN>
 struct TanConsts {
   float D0, k1, r0, h, n, inv2n, lam, mu, kl, km, gcd;
-  float kR1, pR, pA, S, g0, gc2, d2, d, c;   // Tersoff form: f_R exponent, prefactors 1/(S-1), S/(S-1)
+  float kR1, pR, pA, S, g0, d2, d, c;   // Tersoff form: f_R exponent, prefactors 1/(S-1), S/(S-1)
 };
 
 // Raw sums per loss term: 0 Y R, 1 X T + f T B zdot, 2 R (dr Y + rho f), 3 dr (X T + f T B zdot) + rho f T
@@ -391,7 +391,7 @@ __global__ void __launch_bounds__(kTanThreads, 2) tangent_kernel(const TangentPa
       K.mu = k0.w;
       K.lam = -2.f * k2.w;
       K.kR1 = k2.y;
-      K.g0 = k3.x; K.gc2 = k3.y; K.d2 = k3.z; K.gcd = k3.w;
+      K.g0 = k3.x; K.d2 = k3.z; K.gcd = k3.w;
     } else {
       K.D0 = k0.x;
       K.gcd = k1.x;

@@ -90,7 +90,7 @@ __device__ __forceinline__ void sst(T *p, const T &v, int site) {
 template <typename R>
 struct PConsts {
   R D0, k1, k0, mha, beta, h, n, inv2n;
-  R cR, kR1, kR0, hl, g0, gc2, d2, gcd;
+  R cR, kR1, hl, g0, gc2, d2, gcd;
 };
 constexpr int kFormMinimal = 0, kFormTersoff = 1;
 
@@ -98,13 +98,12 @@ constexpr int kFormMinimal = 0, kFormTersoff = 1;
 // zeta is clamped to 1e-30 from below: at zeta = 0 this gives b = 1 to working precision, and b'
 // stays finite; it then only ever multiplies g or g' of the same (vanishing) pairs, so every
 // contribution of a zeta = 0 bond to the forces is exactly zero, as with b' = 0.
-template <typename T>
-__device__ __forceinline__ void bond_order(T zeta, const PConsts<T> &K, T &b, T &bp) {
-  const T z = zeta > T(1e-30f) ? zeta : T(1e-30f);
-  const T zn = ex2(K.n * lg2(z));
-  const T u = T(1.0f) + zn;
+__device__ __forceinline__ void bond_order(float zeta, const PConsts<float> &K, float &b, float &bp) {
+  const float z = zeta > 1e-30f ? zeta : 1e-30f;
+  const float zn = ex2(K.n * lg2(z));
+  const float u = 1.0f + zn;
   b = ex2(K.inv2n * lg2(u));
-  bp = T(-0.5f) * b * zn * rcp(z * u);
+  bp = -0.5f * b * zn * rcp(z * u);
 }
 
 template <typename R>
@@ -499,9 +498,6 @@ __device__ __forceinline__ double ld_cluster(unsigned addr, double) {
   asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr));
   return v;
 }
-__device__ __forceinline__ void st_cluster(unsigned addr, float v) {
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
-}
 __device__ __forceinline__ void st_cluster(unsigned addr, double v) {
   asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
 }
@@ -765,7 +761,7 @@ __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R>
     K.beta = k1.x; K.h = k1.y; K.n = k1.z; K.inv2n = k1.w;
     if constexpr (GEN) {
       const R4 k2 = kc[2], k3 = kc[3];
-      K.cR = k2.x; K.kR1 = k2.y; K.kR0 = k2.z; K.hl = kHalf * k2.w;
+      K.cR = k2.x; K.kR1 = k2.y; K.hl = kHalf * k2.w;
       K.g0 = k3.x; K.gc2 = k3.y; K.d2 = k3.z; K.gcd = k3.w;
     }
   }

@@ -12,9 +12,9 @@ namespace tsf {
 constexpr int kWarp = 32;
 
 // ---------------------------------------------------------------------------------------------
-// Transcendentals. FP32 uses the SFU (MUFU) instructions directly through PTX; FP64 calls the
-// CUDA math library. exp(x) = 2^(x log2 e) is formed by the callers, which fold log2 e into the
-// per-parameter-set constants.
+// Transcendentals in FP32: the SFU (MUFU) instructions directly through PTX. exp(x) = 2^(x log2 e) is
+// formed by the callers, which fold log2 e into the per-parameter-set constants. (FP64: the fixed-point
+// functions of fx64.cuh, and CUDA's math library beyond their ranges and in the plain path.)
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ float ex2(float x) {
   float y;
@@ -31,9 +31,6 @@ __device__ __forceinline__ float rcp(float x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-__device__ __forceinline__ double ex2(double x) { return exp2(x); }
-__device__ __forceinline__ double lg2(double x) { return log2(x); }
-__device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
 
 template <typename R>
 struct Vec4;
