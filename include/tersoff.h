@@ -120,9 +120,9 @@ int tersoff_build_info(tersoff_ctx *ctx, int64_t *ntot, int64_t *nbonds, int32_t
  *  params    device [P][6] double (order of Eq. 16), P >= 1; [P][9] in the Tersoff form
  *            (tersoff_set_form)
  *  precision 32: per-pair arithmetic in FP32; each warp sums its atoms' energy and virial terms in
- *            FP32; the sum of a CTA's per-warp partial sums is their exact sum rounded once to FP64
- *            (fixed-point integer accumulation), and the sums over cluster ranks are FP64 additions,
- *            all in a fixed order; F in float;
+ *            FP32; a CTA's per-warp partial sums are added in FP32 splits (64-bit integers where an
+ *            exponent leaves their range) to an FP64 sum at least as accurate as FP64 additions, and the
+ *            sums over cluster ranks are FP64 additions, all in a fixed order; F in float;
  *            64: everything in FP64, F in double
  *  E         device [P][C] double, total energy (eV)             -- may be NULL
  *  F         device [P][Ntot][3] float or double (see precision) -- may be NULL
@@ -186,7 +186,7 @@ int tersoff_fitness_static(tersoff_ctx *ctx, const double *params, int32_t P,
  * warp and three CTAs per SM) and
  * whether a partly filled last tile runs more atoms per warp -- over whole launches (the best of
  * `reps` timed launches after one warm-up, CUDA events on `stream`), and keeps the fastest in the
- * context. Later tersoff_fitness / tersoff_fitness_static / tersoff_eval calls with the same P use
+ * context. Later tersoff_fitness / tersoff_fitness_static calls with the same P use
  * it until a rebuild changes the neighbour counts. Results of a tuned schedule equal the untuned
  * ones up to the FP32 summation order of the warps' atom groups. Synchronises `stream`.
  *  reps 1..100; best_ms (host, may be NULL) receives the tuned launch time in ms; tried (host, may
@@ -292,9 +292,10 @@ int tersoff_md_export_neighbors(tersoff_ctx *ctx, int32_t *cnt, int32_t *nbr, in
  *    launch while the arguments (pointers, P, weights, precision), the neighbour build's work
  *    schedule and the context's buffers are unchanged; any change re-captures. Calls made while
  *    kernel timing (tersoff_profile) is on, or on a stream that is being captured, launch directly.
- *  TERSOFF_LAUNCH_PDL: the batched and finalize kernels are launched with programmatic stream
- *    serialization, so each may start while its predecessor finishes (it waits before reading the
- *    predecessor's results).
+ *  TERSOFF_LAUNCH_PDL: the fitness's and the gradient's kernels after the preparation (batched, tangent,
+ *    finalize), those of tersoff_md_force from 131,072 atoms on and of tersoff_md_nve are launched with
+ *    programmatic stream serialization, so each may start while its predecessor finishes (it waits
+ *    before reading the predecessor's results).
  * Results are identical in every mode. Returns TERSOFF_E_ARG for a null context or unknown bits. */
 #define TERSOFF_LAUNCH_GRAPHS 1
 #define TERSOFF_LAUNCH_PDL 2

@@ -225,8 +225,8 @@ class Context:
         return 9 if self.form == FORM_TERSOFF else 6
 
     def set_launch_mode(self, graphs: bool = True, pdl: bool = True):
-        """Replay the fitness call's launch sequence from a cached CUDA graph (graphs) and/or launch its
-        kernels with programmatic dependent launch (pdl); both on by default."""
+        """Replay the fitness call's launch sequence from a cached CUDA graph (graphs) and/or launch its kernels, the
+        gradient's and the MD calls' with programmatic dependent launch (pdl); both on by default."""
         self._check(self.lib.tersoff_set_launch_mode(self.h, (LAUNCH_GRAPHS if graphs else 0) | (LAUNCH_PDL if pdl else 0)))
 
     def set_wait_limit(self, spins: int = -1):

@@ -532,8 +532,11 @@ __global__ void __launch_bounds__(kGradFinThreads) grad_finalize_kernel(
 
 // ---------------------------------------------------------------------------------------------
 // Parameter sets per tile of the tangent kernel: the width with the least padded work. Narrow tiles read their
-// geometry per atom slot instead of as broadcasts and run the longest list of their slots, which costs a few
-// per cent; at P = 13 (one Newton iteration) a 16-wide tile does 16 lanes' work instead of 32.
+// geometry per atom slot instead of as broadcasts and run the longest list of their slots; at P = 13 (one Newton
+// iteration) a 16-wide tile does 16 lanes' work instead of 32. What narrow tiles cost, on full ones of 32, 16 and 8 sets
+// (192 sets): 61.0, 63.2 and 65.2 us on 100 cells of 64 atoms, 134, 130 and 157 us on 100 mixed cells; with 96 sets 37.8,
+// 37.4 and 35.8, and 74.9, 73.8 and 87.8 us. The weights 1.08 and 1.15 are at the upper end of the first and about the
+// second, so a narrower tile is taken only where it saves more lanes than that.
 static int tangent_tile(int P) {
   const double c32 = (P + 31) / 32 * 32, c16 = 1.08 * ((P + 15) / 16 * 16), c8 = 1.15 * ((P + 7) / 8 * 8);
   return c32 <= c16 && c32 <= c8 ? 32 : (c16 <= c8 ? 16 : 8);

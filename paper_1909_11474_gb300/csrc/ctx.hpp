@@ -113,7 +113,7 @@ __host__ __device__ inline int pair_slots(int m) { return ((m * (m - 1) / 2) + 3
 
 // A launch bucket: items with the same kernel variant.
 struct Bucket {
-  int mmax;        // 5 or 8: largest neighbour count the variant handles
+  int mmax;        // 4, 6 or 8: largest neighbour count the variant handles (FP64: 8)
   int cluster;     // CTAs per configuration (1 = no cluster)
   int precision;   // 32 or 64
   size_t smem;     // dynamic shared memory per CTA

@@ -6,11 +6,11 @@
 // atom is kept as its in-cell Cartesian position X = u E (FP32; E = the cell edge vectors H_k / nc_k
 // as rows). A bond to an atom of a neighbouring cell (offset o in {-1,0,1}^3) is d = o E + (X_j - X_i),
 // in FP32 and accurate to ~1e-6 A whatever the box size; its image shift is n = kw + m_i - m_j (kw =
-// the periodic wrap of the neighbouring cell). The FP32 d of (j, i) is exactly the negation of that of
-// (i, j), so the two atoms of a pair decide membership alike. Membership uses the FP32 distance where
-// it is farther than a rounding margin from R2, and the exact FP64 test of the batched build
-// otherwise, so the lists equal the batched build's bit for bit; they are sorted to the same (j, n)
-// order.
+// the periodic wrap of the neighbouring cell). Membership uses an FP32 distance (the search forms it from
+// positions relative to a brick's centre) where it is farther than a rounding margin from R2, and the
+// exact FP64 test of the batched build otherwise: every decision is the exact one, whatever the rounding,
+// so the two atoms of a pair agree and the lists equal the batched build's bit for bit; they are sorted to
+// the same (j, n) order. The force kernel's FP32 d of (j, i) is exactly the negation of that of (i, j).
 #include <math.h>
 
 #include <algorithm>
@@ -357,8 +357,8 @@ __device__ __noinline__ void md_search_atom(int N, int M, int i, const double *_
 // Neighbour lists by bricks of 4x4x6 cells, full shell, no atomics: a CTA stages the records of its brick and of the
 // cells around it (6x6x8) in shared memory, as positions x from the brick's centre with q = |x|^2, two records a pair
 // of 16-byte words, so that one atom's test of a pair is two loads and four packed FP32 operations:
-//   t = q_j + (|x_i|^2 - c) - 2 x_i . x_j = |x_j - x_i|^2 - c,   c above the rounding band's upper edge by G.scan_margin,
-// which bounds the rounding of t (a filter: it decides nothing but which records are looked at). One thread per atom of
+//   t = q_j + (|x_i|^2 - c) - 2 x_i . x_j = |x_j - x_i|^2 - c,   c = G.scan_cut, above the rounding band's upper edge by
+// what bounds the rounding of t (a filter: it decides nothing but which records are looked at). One thread per atom of
 // the brick tests the 9 rows (o0, o1) of its shell; the three cells of a row lie consecutively in the stage, so a row is
 // one run of records, taken in blocks of four pairs: the sign bits of t are shifted into a word, whose set bits give the
 // candidates. Members (FP32 below the band, the exact test in it) are inserted into a sorted list in registers as they
@@ -604,7 +604,10 @@ __device__ __forceinline__ double md_block_sum(const double *src, size_t stride,
 // Deterministic in-kernel sum of per-block partials [K][nblk] (FP64; blocks of TH threads): the last block of each
 // group of md_group(nblk) blocks to finish sums its group into [K][ngroups], and the last group to finish sums the
 // groups, both in a fixed order; quantity 0 goes to *out0 and quantity k >= 1 to out_rest[k - 1]. Up to 256 blocks are
-// one group, whose sum is the result: a second level costs a small system ~1.5 us of latency a kernel. The group sums
+// one group, whose sum is the result (an NVE step with one level against groups of 64: FP32 at 108, 172 and 256 blocks
+// 35.0, 42.0 and 47.7 us against 40.4, 45.6 and 51.0; FP64 at 128 and 250 blocks 41.9 and 56.3 against 45.4 and 57.4).
+// Beyond 256 neither is the better one throughout: one level took 3.8 us off a step at 365 blocks and 2.3 at 1,024, and
+// added 1.5 at 432 and 3.0 at 1,458; 666 and 977 within 2 us. The group sums
 // follow the partials; the counters [ngroups + 1] are zero before the launch and left zero by it. The threads that
 // wrote the block's partials have fenced before the call.
 __host__ __device__ inline int md_group(int nblk) { return nblk <= 256 ? 256 : 64; }
@@ -1214,9 +1217,9 @@ int md_prepare(Ctx &c, int N, const double *pos, const double *boxh, const doubl
     }
     esum += std::sqrt(en);
   }
-  // FP32 distance error: the in-cell positions X (at most the sum of the cell edges in size) and the
-  // offset o E, each rounded, then subtracted and added, stay within ~12 ulp of the cell edge
-  // lengths; the band is 128 ulp wide
+  // FP32 distance error: positions from a brick's centre (at most 4 sums of the cell edges in size), the in-cell part and
+  // the cell's offset each rounded, then added and subtracted, stay within ~35 ulp of that sum (on the global-memory path,
+  // from offsets of one cell, within ~12); the band is 128 ulp wide
   const double margin = 128.0 * 1.2e-7 * esum * 2.0 * R2 + 1e-6;
   G.diag = 1;
   for (int a = 0; a < 3; ++a)
@@ -1271,9 +1274,12 @@ int md_prepare(Ctx &c, int N, const double *pos, const double *boxh, const doubl
   r.N = N;
   r.M = M;
   r.precision = precision;
-  // Programmatic launch overlaps a kernel's start with its predecessor's last blocks (512,000 atoms: 150.6 -> 143.1 us a
-  // call) but costs the host about 1.5 us a launch, which a single call of a small system waits for (4,500 atoms: 66 ->
-  // 73 us): large systems take it, and the steps of a run, whose launches run ahead of the device (md_nve sets it)
+  // Programmatic launch overlaps a kernel's start with its predecessor's last blocks (512,000 atoms, FP32: 142.9 -> 135.5 us
+  // a call, back to back). The line was drawn from two sizes, on a first reading of 66 us without it and 73 with it at 4,500
+  // atoms, which later measurements of both sides in turn do not bear out: 512 atoms 39.1 -> 33.2 us, 4,096 38.8 -> 29.4,
+  // 21,952 41.1 -> 38.3, 64,000 53.2 -> 46.5, 125,000 63.1 -> 52.9 (a call waited for by itself: 54 -> 47, 53 -> 45,
+  // 56 -> 50, 67 -> 61, 78 -> 70; FP64 alike or equal). Nothing speaks for the line any more. The steps of a run take
+  // it at every size (md_nve sets it)
   r.pdl = c.pdl && N >= 131072;
   r.nblk = nblk;
   r.fblk = fblk;
