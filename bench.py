@@ -405,7 +405,7 @@ def run_ours(args):
            "e2e": {"value": round(ws * atom_evals * args.steps / t_e2e, 1), "unit": UNIT,
                    "h2d_bytes_per_step": int(h2d), "d2h_bytes_per_step": int(d2h)},
            "build_only": {"ms": round(1e3 * t_build / args.steps, 4),
-                          "note": "neighbour build and FP32 geometry of the 300 cells, counts read back beside it"},
+                          "note": "neighbour build and FP32 geometry of the 300 cells, counts left in pinned host memory"},
            "gpu_launches": int(launches), "roofline": roofline, "measured_peaks": measured, "clocks": clocks,
            "autotune": {"candidates": tuned_tried, "tuned_launch_ms": None if args.schedule else round(tuned_ms, 4),
                         "schedule": ctx.schedule_info(32)}}
