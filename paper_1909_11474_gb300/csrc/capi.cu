@@ -29,6 +29,7 @@ void bump_buffer_generation() { g_buf_gen.fetch_add(1); }
 namespace {
 
 int fail(tersoff_ctx *ctx, int code, const char *fmt, const char *detail = "") {
+  if (code == TERSOFF_E_CUDA) (void)cudaGetLastError();   // reported here: not to the next call's check of its launches
   if (ctx) {
     char buf[512];
     std::snprintf(buf, sizeof(buf), fmt, detail);

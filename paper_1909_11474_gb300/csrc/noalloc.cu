@@ -24,6 +24,7 @@ std::mutex g_scratch_mu;
 size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
 int set_error(tersoff_ctx *ctx, int code, const char *msg) {
+  if (code == TERSOFF_E_CUDA) (void)cudaGetLastError();   // reported here: not to the next call's check of its launches
   if (ctx) ctx->c.err = msg;
   return code;
 }

@@ -724,3 +724,27 @@ def test_schedule_read_back_can_be_set(ctx, precision):
     for x, y in zip(ctx.fitness(params, tg, precision=precision), want):
         assert torch.equal(x, y)
     assert ctx.get_status() == 0
+
+
+def test_a_failed_allocation_is_reported_once(ctx):
+    """A fitness whose residual terms would take 15 TB fails to allocate them and says so; the calls after it, which check
+    their own launches, succeed."""
+    import ctypes
+
+    from paper_1909_11474_gb300 import binding
+    w = I.workload_ga_batch(P=5, C=300)
+    cs = w["configs"]
+    t = targets_to_device({"E": np.full(cs.C, -4.6), "W": np.zeros((cs.C, 6)), "F": np.zeros((cs.Ntot, 3)),
+                           "mask": np.full(cs.C, 7, np.uint8)})
+    params = torch.tensor(w["params"], device="cuda")
+    pos, box = _build(ctx, cs)
+    want = [x.cpu() for x in ctx.fitness(params, t)]
+    Z = torch.empty(5, dtype=torch.float64, device="cuda")
+    tg, wv = ctx._targets(t), (ctypes.c_double * 3)(1, 1, 1)
+    rc = ctx.lib.tersoff_fitness(ctx.h, params.data_ptr(), 2 ** 31 - 1, ctypes.byref(tg), ctypes.addressof(wv), 32,
+                                 Z.data_ptr(), None, None, binding._stream(None))
+    assert rc == binding.E_CUDA and b"memory" in ctx.lib.tersoff_last_error(ctx.h)
+    ctx.build_neighbors(cs.atom_off, pos, box, 2.8, 3.2, 16)
+    for x, y in zip(ctx.fitness(params, t), want):
+        assert torch.equal(x.cpu(), y)
+    assert ctx.get_status() == 0
