@@ -22,7 +22,9 @@
  *    can see on the host (bad arguments, CUDA launch errors) and then records a message retrievable
  *    with tersoff_last_error. Conditions detected inside kernels (neighbour overflow, a wait that
  *    timed out) set bits of a device status word that tersoff_get_status reads.
- *  - No call falls back to the CPU. A context is not thread-safe; use one context per host thread.
+ *  - No call falls back to the CPU. A context is not thread-safe; use one context per host thread. Its
+ *    calls share its workspace: work queued on different streams is ordered by the caller (a neighbour
+ *    build and the call that uses it next excepted, see tersoff_build_neighbors).
  */
 #ifndef TERSOFF_GB300_H
 #define TERSOFF_GB300_H
@@ -43,7 +45,8 @@ enum {
   TERSOFF_E_CUDA = 3,         /* a CUDA runtime call failed                                       */
   TERSOFF_E_NONFINITE = 4,    /* non-finite input positions or box (device status bit 4)          */
   TERSOFF_E_TIMEOUT = 5,      /* a bounded device-side wait gave up (device status bit 8)         */
-  TERSOFF_E_STATE = 6,        /* call made before tersoff_build_neighbors succeeded               */
+  TERSOFF_E_STATE = 6,        /* call made before tersoff_build_neighbors succeeded, or a build
+                                 on a stream under capture                                        */
   TERSOFF_E_UNSUPPORTED = 7   /* an atom has more neighbours than the evaluation kernels handle   */
 };
 
@@ -102,7 +105,8 @@ typedef struct {
  * per atom. Argument errors are returned by this call. Errors found by the build kernel are
  * returned by that next call (and set bits of the status word): an atom with more than max_nbr
  * entries TERSOFF_E_NBR_OVERFLOW (TERSOFF_STATUS_NBR_OVERFLOW), positions or boxes that are not
- * finite TERSOFF_E_NONFINITE. */
+ * finite TERSOFF_E_NONFINITE. A build cannot be part of a captured graph (the host has to see its
+ * counts): on a stream under capture it returns TERSOFF_E_STATE. */
 int tersoff_build_neighbors(tersoff_ctx *ctx, const tersoff_configs *cfg, double R1, double R2,
                             int32_t max_nbr, tersoff_stream stream);
 
